@@ -267,7 +267,7 @@ __device__ __forceinline__ void issue_stage(uint32_t d, uint32_t a_lo, uint32_t 
 // stages, tensor memory four probe tiles), acc_full (a buffer's task is
 // accumulated), acc_empty (its epilogue has read it), mma_done (all MMAs of
 // the CTA completed), task_full / task_empty (the task ring).  Every wait is
-// bounded (wait_or_abort, mbar_wait, wait_counter, wait_smem_count).
+// bounded (wait_or_abort, mbar_wait, wait_counter).
 // ---------------------------------------------------------------------------
 // One task: (expert, row tile, probe group).  For the gate the row tile is
 // 32 hidden units (128 gate rows); for the head it is a 128-row vocabulary
@@ -289,11 +289,11 @@ struct Ctl {
   uint64_t red_bar;                // the head epilogue's rendezvous
   uint64_t mma_done;
   uint64_t task_full[kTaskSlots];  // the fetcher published the slot's task
-  uint64_t task_empty[kTaskSlots]; // every other role has read it
+  uint64_t task_empty[kTaskSlots]; // every other role has read it (the releaser: has released it)
+  uint64_t task_done[kTaskSlots];  // the epilogue warps are done with the slot's task
   int task_gid[kTaskSlots];        // global task index, -1: no more tasks
   int task_t[kTaskSlots];          // its phase
   Task task[kTaskSlots];           // and the task, decoded once by the fetcher
-  int epi_done;                    // epilogue warps' finished tasks (monotonic)
   uint32_t tmem_slot;
   volatile int abort;
 };
@@ -455,24 +455,6 @@ __device__ __forceinline__ int next_task(Ctl* ctl, uint32_t& kt, volatile int* a
   if (release && (threadIdx.x & 31) == 0) mbar_arrive(&ctl->task_empty[sl]);
   ++kt;
   return gid;
-}
-
-// Waits (bounded) until the shared counter reaches `target`; an acquire at
-// CTA scope, so the writes that the counting warps made before their
-// release-add are visible to the caller afterwards.
-__device__ __forceinline__ bool wait_smem_count(int* ctr, int target, volatile int* abort,
-                                                int* status) {
-  const uint32_t addr = smem_u32(ctr);
-  for (uint32_t n = 0; n < (1u << 22); ++n) {
-    int v;
-    asm volatile("ld.acquire.cta.shared::cta.b32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
-    if (v >= target) return true;
-    if ((n & 63u) == 63u && *abort) return false;
-    __nanosleep(32);
-  }
-  *abort = 1;
-  atomicCAS(status, 0, kStatusTimeout);
-  return false;
 }
 
 // Phase counters.  A launch may run several phases; tasks of phase t + 1
@@ -969,8 +951,8 @@ __global__ void __launch_bounds__(kThreads, 1) tc_persistent_kernel(const TcArgs
       // the loader, the MMA issuer, the Z warps (when probes are
       // generated), the epilogue warps and the releaser read every task
       mbar_init(&ctl->task_empty[q], 3 + (do_z ? kZWarps : 0) + kEpiWarps);
+      mbar_init(&ctl->task_done[q], kEpiWarps);
     }
-    ctl->epi_done = 0;
     mbar_fence_init();
   }
   if (warp == 0) tmem_alloc(&ctl->tmem_slot, kTmemCols);
@@ -1139,21 +1121,28 @@ __global__ void __launch_bounds__(kThreads, 1) tc_persistent_kernel(const TcArgs
     // Publishes each task's operand writes (gate) or finished reads (head)
     // on the group's phase counter once the CTA's epilogue warps are done
     // with it: one gpu-scope fence and one add per task, off the epilogue
-    // warps' path.  The epilogue warps count their finished tasks in shared
-    // memory with a CTA-scope release; this warp's acquire of that count,
-    // then its fence, order their writes before the add.
+    // warps' path.  Each task has its own barrier phase (task_done of its
+    // ring slot, one arrival per epilogue warp): with the two accumulator
+    // buffers a warp may already be a task ahead of another, so a plain count
+    // of arrivals could reach a task's total before its last warp is done.
+    // The slot is given back only after the add, so no warp can arrive for
+    // the slot's next task before this one is published.  The wait's acquire,
+    // then the fence, order the epilogue warps' writes before the add.
     uint32_t kt = 0;
     for (int k = 0;; ++k) {
       int t;
       Task T;
-      if (next_task(ctl, kt, abort, status, t, T) < 0) break;
+      if (next_task(ctl, kt, abort, status, t, T, false) < 0) break;
       const size_t c = (size_t)T.e * g.G + T.grp;
-      if (!SOMA_CHECK(c < (size_t)g.n_experts * g.G, status) ||
-          !wait_smem_count(&ctl->epi_done, kEpiWarps * (k + 1), abort, status))
+      const int sl = k % kTaskSlots;
+      const bool fin = wait_or_abort(&ctl->task_done[sl], (uint32_t)(k / kTaskSlots) & 1u, abort,
+                                     status);
+      if (__any_sync(0xffffffffu, !fin) || !SOMA_CHECK(c < (size_t)g.n_experts * g.G, status))
         break;
       if (lane == 0) {
         __threadfence();
         atomicAdd(T.head ? a.hd + c : a.prod + c, kEpiWarps);
+        mbar_arrive(&ctl->task_empty[sl]);
       }
       __syncwarp();
     }
@@ -1259,7 +1248,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_persistent_kernel(const TcArgs
     // 2]) and reads the cell states that phase t - 1 wrote, possibly in
     // another CTA: the fetcher published the task only after acquiring the
     // group's counters of phase t - 1.  After each task it
-    // counts itself done in shared memory, and the releaser publishes the
+    // arrives on the task's done barrier, and the releaser publishes the
     // task on the group's counter.
     const int ew = warp - kEpiWarp0;
     const int q4 = warp & 3;
@@ -1295,8 +1284,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_persistent_kernel(const TcArgs
         tc_fence_before();
         __syncwarp();
         if (lane == 0) {
-          asm volatile("red.release.cta.shared::cta.add.s32 [%0], 1;" ::"r"(smem_u32(&ctl->epi_done))
-                       : "memory");
+          mbar_arrive(&ctl->task_done[k % kTaskSlots]);
           mbar_arrive(&ctl->acc_empty[buf]);
         }
       }
