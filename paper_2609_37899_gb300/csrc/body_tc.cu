@@ -92,8 +92,6 @@ static_assert(kSmE % 1024 == 0 && kSmO1 % 16 == 0 && kSmO3 % 16 == 0 && kSmAcc %
 constexpr uint32_t kTW = 0, kTZ = 64, kTHead = 128, kTHeadLo = 256, kTWloGate = 320,
                    kTWloMlp1 = 384, kTmemCols = 512;
 
-__device__ __forceinline__ float sigm_b(float x) { return __fdividef(1.0f, 1.0f + __expf(-x)); }
-
 __device__ __forceinline__ float gelu_b(float a) {
   return 0.5f * a * (1.f + erff(a * 0.70710678118654752f));
 }
@@ -440,21 +438,21 @@ __global__ void __launch_bounds__(kThreads, 1) body_tc_kernel(const BodyTcArgs a
         for (int k = 0; k < 4; ++k) {
           const float C = Cg[k], Dd = Dg[k];
           if (k == 2) {
-            ap[k] = fmaf(sigm_b(2.f * (C + Dd)), 2.f, -1.f);
-            am[k] = fmaf(sigm_b(2.f * (C - Dd)), 2.f, -1.f);
+            ap[k] = tanh_f(C + Dd);
+            am[k] = tanh_f(C - Dd);
           } else {
-            ap[k] = sigm_b(C + Dd);
-            am[k] = sigm_b(C - Dd);
+            ap[k] = sigmoid_f(C + Dd);
+            am[k] = sigmoid_f(C - Dd);
           }
         }
         const float cp = fmaf(ap[1], cst[b][0], ap[0] * ap[2]);
         const float cm = fmaf(am[1], cst[b][1], am[0] * am[2]);
         cst[b][0] = cp;
         cst[b][1] = cm;
-        const float hp = ap[3] * fmaf(sigm_b(2.f * cp), 2.f, -1.f);
-        const float hm = am[3] * fmaf(sigm_b(2.f * cm), 2.f, -1.f);
+        float hsum, hdif;
+        h_sum_diff(ap[3], tanh_f(cp), am[3], tanh_f(cm), hsum, hdif);
         const int U = 8 * q4 + u8;
-        const float hb = 0.5f * (hp + hm), hd = 0.5f * (hp - hm);
+        const float hb = 0.5f * hsum, hd = 0.5f * hdif;
         store_split(o1, 64, bseq, kD + U, hb, hd * inv_eps);
         xbar[bseq * kD + U] += hb;
         dx[bseq * kD + U] += hd;
@@ -612,8 +610,8 @@ __global__ void __launch_bounds__(kThreads, 1) body_tc_kernel(const BodyTcArgs a
         float sp_ = 0.f, sm_ = 0.f;
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-          sp_ += __expf(lp[k] - mp);
-          sm_ += __expf(lm[k] - mm);
+          sp_ += exp_term(lp[k] - mp);
+          sm_ += exp_term(lm[k] - mm);
         }
 #pragma unroll
         for (int o = 4; o < 32; o <<= 1) {

@@ -101,8 +101,6 @@ __device__ __forceinline__ uint32_t natural_to_raw(uint32_t n) {
   return compact16(n) | (compact16(n >> 1) << 16);
 }
 
-__device__ __forceinline__ float sigm(float x) { return __fdividef(1.0f, 1.0f + __expf(-x)); }
-
 // Row blocks (units of Bp) of probe p inside an operand group tile and the
 // accumulator columns (units of Bp) of its C and D parts; see the header.
 __host__ __device__ __forceinline__ int row_mean(int p) { return p == 0 ? 1 : 4; }
@@ -685,11 +683,11 @@ __device__ void gate_finish(const TcArgs& a, const Phase& ph, const Task& T, uin
           const float ap = __uint_as_float(vc[h][k]) + G.bias[k];
           const float am = __uint_as_float(vd[h][k]) + G.bias[k];
           if (k == 2) {
-            actp[k] = fmaf(sigm(2.f * ap), 2.f, -1.f);
-            actm[k] = fmaf(sigm(2.f * am), 2.f, -1.f);
+            actp[k] = tanh_f(ap);
+            actm[k] = tanh_f(am);
           } else {
-            actp[k] = sigm(ap);
-            actm[k] = sigm(am);
+            actp[k] = sigmoid_f(ap);
+            actm[k] = sigmoid_f(am);
           }
         }
       } else {
@@ -698,18 +696,19 @@ __device__ void gate_finish(const TcArgs& a, const Phase& ph, const Task& T, uin
           const float C = __uint_as_float(vc[h][k]) + G.bias[k];
           const float D = fmaf(eps, __uint_as_float(vd[h][k]), G.dbias[k]);
           if (k == 2) {  // g: tanh(x) = 2 sigmoid(2x) - 1
-            actp[k] = fmaf(sigm(2.f * (C + D)), 2.f, -1.f);
-            actm[k] = fmaf(sigm(2.f * (C - D)), 2.f, -1.f);
+            actp[k] = tanh_f(C + D);
+            actm[k] = tanh_f(C - D);
           } else {
-            actp[k] = sigm(C + D);
-            actm[k] = sigm(C - D);
+            actp[k] = sigmoid_f(C + D);
+            actm[k] = sigmoid_f(C - D);
           }
         }
       }
       const float cp = fmaf(actp[1], G.cprev[j][h].x, actp[0] * actp[2]);
       const float cm = fmaf(actm[1], G.cprev[j][h].y, actm[0] * actm[2]);
-      const float hp = actp[3] * fmaf(sigm(2.f * cp), 2.f, -1.f);
-      const float hm = actm[3] * fmaf(sigm(2.f * cm), 2.f, -1.f);
+      const float tp = tanh_f(cp), tm = tanh_f(cm);
+      float hsum, hdif;
+      h_sum_diff(actp[3], tp, actm[3], tm, hsum, hdif);
       const int b = b0 + 4 * h + bq;
       const size_t tile_off = (size_t)(out_tile - ph.op_out);
       if (unit_ok &&
@@ -722,18 +721,17 @@ __device__ void gate_finish(const TcArgs& a, const Phase& ph, const Task& T, uin
           // h of the two blocks into their own rows (the W product's rows)
           if (inf_seq(g, T.grp, col_c(p), b) < s.B)
             *reinterpret_cast<__half*>(out_tile + kmajor_offset(rM + b, kk, kKt)) =
-                __float2half_rn(hp);
+                __float2half_rn(actp[3] * tp);
           if (inf_seq(g, T.grp, col_d(p), b) < s.B)
             *reinterpret_cast<__half*>(out_tile + kmajor_offset(rD + b, kk, kKt)) =
-                __float2half_rn(hm);
+                __float2half_rn(actm[3] * tm);
         } else if (b < s.B) {
-          const float dh = hp - hm;
           *reinterpret_cast<__half*>(out_tile + kmajor_offset(rM + b, kk, kKt)) =
-              __float2half_rn(0.5f * (hp + hm));
+              __float2half_rn(0.5f * hsum);
           *reinterpret_cast<__half*>(out_tile + kmajor_offset(rD + b, kk, kKt)) =
-              __float2half_rn(dh * half_inv_eps);
+              __float2half_rn(hdif * half_inv_eps);
           *reinterpret_cast<__half*>(out_tile + kmajor_offset(rE + b, kk, kKt)) =
-              __float2half_rn(dh * half_eps);
+              __float2half_rn(hdif * half_eps);
         }
       }
     }
@@ -833,8 +831,8 @@ __device__ bool head_epilogue(const TcArgs& a, const Phase& ph, const Task& T, u
       float sp = 0.f, sm_ = 0.f;
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
-        sp += __expf(lp[k] - mp);
-        sm_ += __expf(lm[k] - mm);
+        sp += exp_term(lp[k] - mp);
+        sm_ += exp_term(lm[k] - mm);
       }
 #pragma unroll
       for (int o = 4; o < 32; o <<= 1) {
@@ -1674,6 +1672,8 @@ size_t kernel_smem_bytes(const TcGeom& g) {
   return (size_t)kStages * stage_layout(g).bytes + 1024 + red + 1024;
 }
 
+}  // namespace
+
 int sm_count() {
   static int cached[64] = {0};
   int dev = 0;
@@ -1685,8 +1685,6 @@ int sm_count() {
   }
   return cached[dev];
 }
-
-}  // namespace
 
 TcGeom make_tc_geom(const Layout& lay, int n_experts, int n_pert, int B, int T, int B_mem) {
   TcGeom g;

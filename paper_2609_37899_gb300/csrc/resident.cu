@@ -47,8 +47,6 @@ constexpr int kResMaxBp = 32;
 constexpr size_t kResMaxSmem = 220 * 1024;
 constexpr uint32_t kLboRes = 128;  // bytes between core matrices along K
 
-__device__ __forceinline__ float sigm_res(float x) { return __fdividef(1.0f, 1.0f + __expf(-x)); }
-
 struct ResGeom {
   int E, H, Ek, Hk, K, MTg, Bp, B, T;
   uint32_t wg, zg, wo, zo, op, opsz, emb, dx, red, ylog, acc, ctl, bytes;  // shared-memory offsets
@@ -375,26 +373,26 @@ __global__ void __launch_bounds__(kResThreads, 1) res_kernel(const ResArgs a) {
               const float C = fmaf(eps2, __uint_as_float(zd[h][k]), __uint_as_float(wv[h][k])) + bias[k];
               const float D = fmaf(eps, __uint_as_float(wd[h][k]) + __uint_as_float(zv[h][k]), dbias[k]);
               if (k == 2) {
-                actp[k] = fmaf(sigm_res(2.f * (C + D)), 2.f, -1.f);
-                actm[k] = fmaf(sigm_res(2.f * (C - D)), 2.f, -1.f);
+                actp[k] = tanh_f(C + D);
+                actm[k] = tanh_f(C - D);
               } else {
-                actp[k] = sigm_res(C + D);
-                actm[k] = sigm_res(C - D);
+                actp[k] = sigmoid_f(C + D);
+                actm[k] = sigmoid_f(C - D);
               }
             }
             const float cp = fmaf(actp[1], cst[c][h][0], actp[0] * actp[2]);
             const float cm = fmaf(actm[1], cst[c][h][1], actm[0] * actm[2]);
             cst[c][h][0] = cp;
             cst[c][h][1] = cm;
-            const float hp = actp[3] * fmaf(sigm_res(2.f * cp), 2.f, -1.f);
-            const float hm = actm[3] * fmaf(sigm_res(2.f * cm), 2.f, -1.f);
+            float hsum, hdif;
+            h_sum_diff(actp[3], tanh_f(cp), actm[3], tanh_f(cm), hsum, hdif);
             const int b = b0 + 4 * h + bq;
             if (unit_ok && b < g.B &&
                 SOMA_CHECK(kmajor_offset(g.Bp + b, g.Ek + U, g.K) + 2 <= g.opsz, a.status)) {
               *reinterpret_cast<__half*>(smem + g.op + nxt * g.opsz + kmajor_offset(b, g.Ek + U, g.K)) =
-                  __float2half_rn(0.5f * (hp + hm));
+                  __float2half_rn(0.5f * hsum);
               *reinterpret_cast<__half*>(smem + g.op + nxt * g.opsz + kmajor_offset(g.Bp + b, g.Ek + U, g.K)) =
-                  __float2half_rn((hp - hm) * half_inv_eps);
+                  __float2half_rn(hdif * half_inv_eps);
             }
           }
         }
@@ -453,8 +451,8 @@ __global__ void __launch_bounds__(kResThreads, 1) res_kernel(const ResArgs a) {
         float sp = 0.f, sm_ = 0.f;
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-          sp += __expf(lp[k] - mp);
-          sm_ += __expf(lm[k] - mm);
+          sp += exp_term(lp[k] - mp);
+          sm_ += exp_term(lm[k] - mm);
         }
 #pragma unroll
         for (int o = 4; o < 32; o <<= 1) {

@@ -15,6 +15,9 @@ namespace soma {
 void trace_begin(int kind, cudaStream_t stream);
 void trace_end(int kind, cudaStream_t stream);
 
+// SMs of the current device.
+int sm_count();
+
 
 // ---- tensor-core path ------------------------------------------------------
 // Geometry of one sweep on the tensor cores.  K of the gate GEMM is

@@ -190,6 +190,14 @@ __device__ __forceinline__ void mma_f16_ts_lohi(uint32_t d_tmem, uint32_t a_tmem
       : "memory");
 }
 
+// 8 consecutive 32-bit columns of this thread's TMEM lane <- r[0..7].
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t* r) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(taddr),
+               "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]),
+               "r"(r[7])
+               : "memory");
+}
+
 // 16 consecutive 32-bit columns of this thread's TMEM lane <- r[0..15].
 __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t* r) {
   asm volatile(
@@ -281,6 +289,46 @@ __device__ __forceinline__ uint32_t pm_pair(uint32_t raw, uint32_t mag2) {
   static_assert(J >= 0 && J < 16, "pair index");
   return ((raw << (15 - J)) & 0x80008000u) | mag2;
 }
+
+// ----------------------------------------------------------- activations --
+// 2^x and 1 / x on the special-function unit, subnormals as zero.  The
+// sigmoids and softmax terms below add the power to a value of at least 1, so
+// a subnormal power (which __expf keeps, at the price of a range test and two
+// scalings per call) never shows: checked bit for bit against __expf and
+// __fdividef over every float.  An epilogue spends most of its issue slots
+// here: the cells' ten activations per (unit, sequence) went from about 13
+// instructions each to four.
+__device__ __forceinline__ float ex2_ftz(float x) {
+  float r;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float rcp_ftz(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+constexpr float kLog2e = 1.4426950408889634f;  // exp(x) = 2^(x log2 e)
+
+__device__ __forceinline__ float sigmoid_f(float x) {
+  return rcp_ftz(1.0f + ex2_ftz(x * -kLog2e));
+}
+// tanh(x) = 2 sigmoid(2x) - 1
+__device__ __forceinline__ float tanh_f(float x) {
+  return fmaf(rcp_ftz(1.0f + ex2_ftz(x * (-2.0f * kLog2e))), 2.f, -1.f);
+}
+// h+- = o+- tanh(c+-) of the two signs as their sum and difference, from o and
+// tanh(c) of each: the + product enters exactly, the - product rounded (one
+// contraction of the two possible, written out so that every kernel has the
+// same).
+__device__ __forceinline__ void h_sum_diff(float op, float tp, float om, float tm, float& sum,
+                                           float& dif) {
+  const float hm = __fmul_rn(om, tm);
+  sum = fmaf(op, tp, hm);
+  dif = fmaf(op, tp, -hm);
+}
+// exp(x), x <= 0, for sums that hold a term of at least 1
+__device__ __forceinline__ float exp_term(float x) { return ex2_ftz(x * kLog2e); }
 
 // Gate tile rows: a 128-row tile covers 32 hidden units.  Tile row r lies in
 // TMEM lane quarter r / 32 and holds gate (r / 8) % 4 of unit 8 (r / 32) +
