@@ -264,6 +264,14 @@ __device__ __forceinline__ void tmem_ld_16x128b(uint32_t taddr, uint32_t& r0, ui
                : "r"(taddr));
 }
 
+// Two repetitions: (r0, r1) of columns c + l % 4 and (r2, r3) of columns c + 4 + l % 4.
+__device__ __forceinline__ void tmem_ld_16x128b_x2(uint32_t taddr, uint32_t& r0, uint32_t& r1,
+                                                   uint32_t& r2, uint32_t& r3) {
+  asm volatile("tcgen05.ld.sync.aligned.16x128b.x2.b32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
+               : "r"(taddr));
+}
+
 __device__ __forceinline__ void tmem_wait_ld() {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
