@@ -71,11 +71,16 @@ constexpr int kFetchWarp = 2;    // takes tasks and acquires their phase counter
 constexpr int kRelWarp = 3;      // publishes finished tasks on the phase counters
 constexpr int kZWarp0 = 4;       // Z generators: a multiple of 4 (TMEM lane quarters)
 constexpr int kZWarps = 8;       // (probe, lane quarter)
-constexpr int kEpiWarp0 = kZWarp0 + kZWarps;
-constexpr int kEpiWarps = 8;     // (probe, lane quarter)
-constexpr int kEpiProbeStep = kEpiWarps / 4;  // head: warp group eg runs probes eg, eg + 2, ...
-constexpr int kThreads = (kEpiWarp0 + kEpiWarps) * 32;
-static_assert(kZWarp0 % 4 == 0 && kEpiWarp0 % 4 == 0, "warp w reads TMEM lane quarter w % 4");
+// Epilogue warps EPI (a multiple of 8: probe or sequence share, lane quarter):
+// 16 in the unperturbed layout, which has no probe tiles and takes the
+// generators' warps; 8 or 16 in the perturbed one (see epi_warps_for).
+constexpr int kInfEpi = 16;
+template <bool INF, int EPI>
+struct Warps {
+  static constexpr int epi0 = INF ? kZWarp0 : kZWarp0 + kZWarps;
+  static constexpr int threads = (epi0 + EPI) * 32;
+};
+static_assert(kZWarp0 % 4 == 0 && kZWarps % 4 == 0, "warp w reads TMEM lane quarter w % 4");
 constexpr int kTaskSlots = 4;               // tasks a CTA's fetcher publishes ahead of the others
 constexpr int kKt = 64;                     // K per stage (fp16 elements)
 constexpr uint32_t kTileA = 128 * kKt * 2;  // one 128-row A tile per stage
@@ -255,9 +260,11 @@ __device__ __forceinline__ void issue_stage(uint32_t d, uint32_t a_lo, uint32_t 
 //                 words of the sweep's table into the fp16 +-1 row of its
 //                 probe tile and stores it into the slot's TMEM columns
 //                 (lane = row);
-//   warps 12..19  epilogue: reads a finished accumulator buffer while the
-//                 MMAs of the next task fill the other one; warp w reads the
-//                 TMEM lanes of quarter w % 4 for probe group (w - 12) / 4.
+//   warps 12 ..   epilogue (EPI warps): reads a finished accumulator buffer while
+//                 the MMAs of the next task fill the other one; warp w reads the
+//                 TMEM lanes of quarter w % 4 for its share of the group's
+//                 probes and sequences (epi_share).  In the unperturbed layout
+//                 there are no generators and the epilogue starts at warp 4.
 // Barriers: full (the slot's copies landed and its Z tiles are stored: the
 // loader's arrival with the copies' bytes and one arrival per Z warp, so the
 // issuer waits once per stage), slot_free (the slot's MMAs are done), z_free
@@ -457,17 +464,16 @@ __device__ __forceinline__ int next_task(Ctl* ctl, uint32_t& kt, volatile int* a
 
 // Phase counters.  A launch may run several phases; tasks of phase t + 1
 // start on the groups that phase t has finished, without a grid-wide
-// barrier.  Per (expert, group): prod counts the writes finished into the
-// group's operand (one per epilogue warp of a gate task), hd the head tasks
-// finished (one per epilogue warp).
+// barrier.  Per (expert, group): prod counts the gate tasks finished (their
+// writes into the group's operand), hd the head tasks.
 // Through phase t (inclusive):
 __device__ __forceinline__ int prod_target(const TcArgs& a, int t) {
   if (t < 0) return 0;
   const int gate_phases = min(t, a.sw.T - 1) + 1;
-  return kEpiWarps * a.g.MT * gate_phases;
+  return a.g.MT * gate_phases;
 }
 __device__ __forceinline__ int hd_target(const TcArgs& a, int t) {
-  return t < 1 ? 0 : kEpiWarps * 2 * t;
+  return t < 1 ? 0 : 2 * t;
 }
 
 // Waits (bounded) until *ctr >= target; lane 0 polls for the warp.  The
@@ -555,10 +561,23 @@ __host__ __device__ __forceinline__ size_t zbits_row(const TcGeom& g, int e, int
   return (((size_t)e * g.n_pert + probe) * zbits_stages(g) + ts) * kZRows;
 }
 
+// The share of an epilogue warp: TMEM lane quarter w % 4 of one probe p, and of
+// its sequence chunks those c with c % parts == part.  With P = 2 the warp groups
+// eg = ew / 4 alternate between the probes, with P = 1 all run probe 0.
+struct EpiShare {
+  int p, part, parts;
+};
+template <int EPI>
+__device__ __forceinline__ EpiShare epi_share(const TcGeom& g, int ew) {
+  constexpr int groups = EPI / 4;
+  const int eg = ew >> 2;
+  if (g.P == 2) return {eg & 1, eg >> 1, groups / 2};
+  return {0, eg, groups};
+}
+
 // Gate epilogue of one task for one warp of TMEM lane quarter q4 (units
-// 8 q4 .. 8 q4 + 7 of the tile).  With P = 2 the warps of group eg = 0, 1 run
-// probe eg; with P = 1 both groups run probe 0 and split its 8-sequence
-// chunks.  Thread l runs the cells of unit l / 4 for sequences b0 + l % 4 and
+// 8 q4 .. 8 q4 + 7 of the tile), 8 sequences per chunk.  Thread l runs the
+// cells of unit l / 4 for sequences b0 + l % 4 and
 // b0 + 4 + l % 4 of each of its chunks, both signs, in fp32: 16x128b loads
 // give it all four gates of its unit (gate-major rows), so no data moves
 // between threads.  It writes the three operand rows of its (unit,
@@ -568,58 +587,42 @@ __host__ __device__ __forceinline__ size_t zbits_row(const TcGeom& g, int e, int
 // gate_prepare runs before the accumulator is ready: it loads the bias, its
 // probe signs and the previous cell states, so that their latency overlaps
 // the task's MMAs.
-constexpr int kEpiMaxChunks = 4;  // Bp <= 32 with P = 2; Bp <= 64 split over two groups with P = 1
-
+// Chunks of one warp: Bp <= 32 with P = 2, Bp <= 64 with P = 1.
+template <int EPI>
 struct GatePre {
+  static constexpr int chunks = 32 / EPI;
   float bias[4], dbias[4];
-  float2 cprev[kEpiMaxChunks][2];
+  float2 cprev[chunks][2];
   int p, c0, cstep;
   bool on;
 };
 
-template <bool INF>
+template <bool INF, int EPI>
 __device__ __forceinline__ void gate_prepare(const TcArgs& a, const Phase& ph, const Task& T,
-                                             int q4, int eg, GatePre& G) {
+                                             int q4, int ew, GatePre<EPI>& G) {
   const TcGeom& g = a.g;
   const Sweep& s = a.sw;
   const Layout& L = s.lay;
   const int lane = threadIdx.x & 31;
   const int H = g.H;
-  G.p = g.P == 2 ? eg : 0;
-  G.c0 = g.P == 2 ? 0 : eg;
-  G.cstep = g.P == 2 ? 1 : 2;
+  const EpiShare sh = epi_share<EPI>(g, ew);
+  G.p = sh.p;
+  G.c0 = sh.part;
+  G.cstep = sh.parts;
   G.on = G.p < T.p_valid;
   if (!G.on) return;
   const int i = T.grp * g.P + G.p;
   const ProbeKey pk = make_probe_key(s.seed, s.step, (uint32_t)T.e, (uint32_t)i);
   const float eps = s.eps;
   const float* th = s.params + (int64_t)T.e * L.P;
-  // bias and its probe sign for the row in this lane's TMEM lane, handed to
-  // the threads that run that row's unit
-  float bias_r = 0.f, dbias_r = 0.f;
-  {
-    const int Ur = 32 * T.m + tile_unit(32 * q4 + lane);
-    const int64_t pb = L.b + (int64_t)tile_gate(32 * q4 + lane) * H + Ur;
-    if (Ur < H && SOMA_CHECK((size_t)(T.e * L.P + pb) < a.n_params, a.status)) {
-      bias_r = th[pb];
-      if (eps != 0.f) {
-        const ProbeBits zb = probe_bits(pk, pb, s.sparse);
-        dbias_r = eps_z(zb.neg & 1u, zb.act & 1u, eps);
-      }
-    }
-  }
+  // the cell states first: their loads are the longest
   const int u8 = lane >> 2, bq = lane & 3;
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    G.bias[k] = __shfl_sync(0xffffffffu, bias_r, 8 * k + u8);
-    G.dbias[k] = __shfl_sync(0xffffffffu, dbias_r, 8 * k + u8);
-  }
   const int U = 32 * T.m + 8 * q4 + u8;
   const float2* cell = reinterpret_cast<const float2*>(a.cst) +
                        (((int64_t)T.e * cst_lanes_of<INF>(g) + i) * g.Hp + U) * (int64_t)g.Bp;
   const bool load = U < H && ph.t_gate > 0;
 #pragma unroll
-  for (int j = 0; j < kEpiMaxChunks; ++j) {
+  for (int j = 0; j < GatePre<EPI>::chunks; ++j) {
     const int b0 = 8 * (G.c0 + j * G.cstep);
     G.cprev[j][0] = G.cprev[j][1] = make_float2(0.f, 0.f);
     if (load && b0 < g.Bp &&
@@ -629,11 +632,30 @@ __device__ __forceinline__ void gate_prepare(const TcArgs& a, const Phase& ph, c
       G.cprev[j][1] = cell[b0 + 4 + bq];
     }
   }
+  // bias and its probe sign for the row in this lane's TMEM lane, handed to
+  // the threads that run that row's unit
+  float bias_r = 0.f, dbias_r = 0.f;
+  {
+    const int Ur = 32 * T.m + tile_unit(32 * q4 + lane);
+    const int64_t pb = L.b + (int64_t)tile_gate(32 * q4 + lane) * H + Ur;
+    if (Ur < H && SOMA_CHECK((size_t)(T.e * L.P + pb) < a.n_params, a.status)) {
+      bias_r = th[pb];
+      if (eps != 0.f) {
+        const ProbeBits zb = probe_bit(pk, pb, s.sparse);
+        dbias_r = eps_z(zb.neg, zb.act, eps);
+      }
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    G.bias[k] = __shfl_sync(0xffffffffu, bias_r, 8 * k + u8);
+    G.dbias[k] = __shfl_sync(0xffffffffu, dbias_r, 8 * k + u8);
+  }
 }
 
-template <bool INF>
+template <bool INF, int EPI>
 __device__ void gate_finish(const TcArgs& a, const Phase& ph, const Task& T, uint32_t tacc,
-                            int q4, const GatePre& G) {
+                            int q4, const GatePre<EPI>& G) {
   if (!G.on) return;
   const TcGeom& g = a.g;
   const Sweep& s = a.sw;
@@ -658,7 +680,7 @@ __device__ void gate_finish(const TcArgs& a, const Phase& ph, const Task& T, uin
   const uint32_t cC = (uint32_t)(col_c(p) * g.Bp), cD = (uint32_t)(col_d(p) * g.Bp);
   const int rM = row_mean(p) * g.Bp, rD = row_dhat(p) * g.Bp, rE = row_e2(p) * g.Bp;
 #pragma unroll
-  for (int j = 0; j < kEpiMaxChunks; ++j) {
+  for (int j = 0; j < GatePre<EPI>::chunks; ++j) {
     const int b0 = 8 * (G.c0 + j * G.cstep);
     if (b0 >= g.Bp) break;
     // [seq half][gate]: C (W vbar + eps^2 Z dhat) and D (W dhat + Z vbar)
@@ -739,13 +761,72 @@ __device__ void gate_finish(const TcArgs& a, const Phase& ph, const Task& T, uin
 }
 
 // Head epilogue of one task: logits +- of the 32 vocabulary rows of the
-// warp's lane quarter for each probe the warp runs.  16x128b loads give
-// thread l four rows (l / 4 + {0, 8, 16, 24}) of sequence b0 + l % 4, so
-// the per-(sequence, sign) max and sum-exp over the quarter reduce four rows
-// in registers and then across the eight threads of that sequence (three
-// shuffle rounds).  The four quarters of the half merge through shared
-// memory (`red`, [P][Bp][2][4]); the thread holding the target byte's row
-// writes the target logit.
+// warp's lane quarter for the warp's share of the probe's sequences, in groups
+// of four.  16x128b loads give thread l four rows (l / 4 + {0, 8, 16, 24}) of
+// sequence b0 + l % 4, so the per-(sequence, sign) max and sum-exp over the
+// quarter reduce four rows in registers and then across the eight threads of
+// that sequence (three shuffle rounds); two groups go at a time.  The four
+// quarters of the half merge through shared memory (`red`, [P][Bp][2][4]); the
+// thread holding the target byte's row writes the target logit.
+//
+// head_prepare runs before the accumulator is ready: biases, their probe signs
+// and the target bytes.  Loading a target in the loop cost an L2 round trip
+// per group (the acquire of the phase counters empties L1): 13,000 to 20,000
+// cycles per head task against about 4,000 for a gate task's epilogue.
+constexpr int kHeadMaxGroups = 8;  // 4-sequence groups of one warp (INF: two targets each)
+
+struct HeadPre {
+  float bo[4], dbo[4];
+  uint32_t tgt[4];  // target bytes, one per group (INF: per group and block)
+  EpiShare sh;
+  bool on;
+};
+
+template <bool INF, int EPI>
+__device__ __forceinline__ void head_prepare(const TcArgs& a, const Phase& ph, const Task& T,
+                                             int q4, int ew, HeadPre& G) {
+  const TcGeom& g = a.g;
+  const Sweep& s = a.sw;
+  const Layout& L = s.lay;
+  const int lane = threadIdx.x & 31;
+  const int bq = lane & 3, r4 = lane >> 2;
+  G.sh = epi_share<EPI>(g, ew);
+  G.on = G.sh.p < T.p_valid;
+  if (!G.on) return;
+  const float* th = s.params + (int64_t)T.e * L.P;
+  const int vq = 128 * T.m + 32 * q4;  // first vocabulary row of the quarter
+  const float bo_r =
+      SOMA_CHECK((size_t)(T.e * L.P + L.b_out + vq + lane) < a.n_params, a.status)
+          ? th[L.b_out + vq + lane]
+          : 0.f;
+  const int i = T.grp * g.P + G.sh.p, t = ph.t_head;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) G.tgt[k] = 0u;
+#pragma unroll
+  for (int j = 0; j < kHeadMaxGroups; ++j) {
+    const int b = 4 * (G.sh.part + (INF ? j >> 1 : j) * G.sh.parts) + bq;
+    // unperturbed: the sequences of blocks col_c(p) and col_d(p)
+    const int q = INF ? inf_seq(g, T.grp, j & 1 ? col_d(G.sh.p) : col_c(G.sh.p), b) : b;
+    if (b < g.Bp && q < s.B) {
+      const int64_t o = seq_offset(s, T.e, INF ? 0 : i, q) + t + 1;
+      if (SOMA_CHECK((size_t)o < a.n_bytes, a.status))
+        G.tgt[j >> 2] |= (uint32_t)s.bytes[o] << (8 * (j & 3));
+    }
+  }
+  float dbo_r = 0.f;
+  if (s.eps != 0.f) {
+    const ProbeKey pk = make_probe_key(s.seed, s.step, (uint32_t)T.e, (uint32_t)i);
+    const ProbeBits zb = probe_bit(pk, L.b_out + vq + lane, s.sparse);
+    dbo_r = eps_z(zb.neg, zb.act, s.eps);
+  }
+  // rows of this thread: vq + r4 + 8 k, k = 0..3 (k = 2 h + reg)
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    G.bo[k] = __shfl_sync(0xffffffffu, bo_r, r4 + 8 * k);
+    G.dbo[k] = __shfl_sync(0xffffffffu, dbo_r, r4 + 8 * k);
+  }
+}
+
 // Rendezvous of the epilogue warps around the head's reduction buffer: a
 // bounded wait on an mbarrier (count: one arrival per epilogue warp), so a
 // warp that has left after an abort makes the others time out instead of
@@ -760,131 +841,130 @@ __device__ __forceinline__ bool epi_rendezvous(uint64_t* bar, uint32_t* use, vol
   return ok;
 }
 
-template <bool INF>
+template <bool INF, int EPI>
 __device__ bool head_epilogue(const TcArgs& a, const Phase& ph, const Task& T, uint32_t tacc,
-                              int q4, int ew, float2* red, uint64_t* red_bar, uint32_t* red_use,
-                              volatile int* abort) {
+                              int q4, int ew, const HeadPre& G, float2* red, uint64_t* red_bar,
+                              uint32_t* red_use, volatile int* abort) {
   const TcGeom& g = a.g;
   const Sweep& s = a.sw;
-  const Layout& L = s.lay;
   const int lane = threadIdx.x & 31;
   const float eps = s.eps;
-  const bool do_z = eps != 0.f;
-  const float* th = s.params + (int64_t)T.e * L.P;
-  const int vq = 128 * T.m + 32 * q4;  // first vocabulary row of the quarter
-  const float bo_r =
-      SOMA_CHECK((size_t)(T.e * L.P + L.b_out + vq + lane) < a.n_params, a.status)
-          ? th[L.b_out + vq + lane]
-          : 0.f;
+  const int vq = 128 * T.m + 32 * q4;
   const int t = ph.t_head;
   const int bq = lane & 3, r4 = lane >> 2;
-  // rows of this thread: vq + r4 + 8 k, k = 0..3 (k = 2 h + reg)
-  float bo[4];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) bo[k] = __shfl_sync(0xffffffffu, bo_r, r4 + 8 * k);
   const uint32_t tq = tacc + ((uint32_t)(32 * q4) << 16);
   const uint32_t tq2 = tq + (16u << 16);
-  for (int p = ew >> 2; p < g.P; p += kEpiProbeStep) {
-    if (p >= T.p_valid) continue;
-    const int i = T.grp * g.P + p;
-    float dbo[4] = {0.f, 0.f, 0.f, 0.f};
-    if (do_z) {
-      const ProbeKey pk = make_probe_key(s.seed, s.step, (uint32_t)T.e, (uint32_t)i);
-      const ProbeBits zb = probe_bits(pk, L.b_out + vq + lane, s.sparse);
-      const float dbo_r = eps_z(zb.neg & 1u, zb.act & 1u, eps);
-#pragma unroll
-      for (int k = 0; k < 4; ++k) dbo[k] = __shfl_sync(0xffffffffu, dbo_r, r4 + 8 * k);
-    }
+  if (G.on) {
+    const int p = G.sh.p, i = T.grp * g.P + p;
     // perturbed: lanes (e, i, +) and (e, i, -) for sequence b; unperturbed:
     // lane (e, 0, +) for the sequences of blocks col_c(p) and col_d(p)
     const int64_t lane_plus = INF ? (int64_t)T.e * 2 : ((int64_t)T.e * s.n_pert + i) * 2;
     const uint32_t cC = (uint32_t)(col_c(p) * g.Bp), cD = (uint32_t)(col_d(p) * g.Bp);
-    for (int b0 = 0; b0 < g.Bp; b0 += 4) {
-      // [k]: C and D of row r4 + 8 k, sequence b0 + bq
-      uint32_t vc[4], vd[4];
-      const uint32_t cw = (uint32_t)b0;
-      tmem_ld_16x128b(tq + cC + cw, vc[0], vc[1]);
-      tmem_ld_16x128b(tq2 + cC + cw, vc[2], vc[3]);
-      tmem_ld_16x128b(tq + cD + cw, vd[0], vd[1]);
-      tmem_ld_16x128b(tq2 + cD + cw, vd[2], vd[3]);
+    const int step = 4 * G.sh.parts;
+#pragma unroll
+    for (int j0 = 0; j0 < (INF ? kHeadMaxGroups / 2 : kHeadMaxGroups); j0 += 2) {
+      const int b0 = 4 * G.sh.part + j0 * step;
+      if (b0 >= g.Bp) break;
+      // [group][k]: logits of row r4 + 8 k, sequence b0 + h step + bq; a second
+      // group past Bp repeats the first
+      float lp[2][4], lm[2][4], mp[2], mm[2], sp[2], sm_[2];
+      uint32_t vc[2][4], vd[2][4];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const uint32_t cw = (uint32_t)(b0 + h * step < g.Bp ? b0 + h * step : b0);
+        tmem_ld_16x128b(tq + cC + cw, vc[h][0], vc[h][1]);
+        tmem_ld_16x128b(tq2 + cC + cw, vc[h][2], vc[h][3]);
+        tmem_ld_16x128b(tq + cD + cw, vd[h][0], vd[h][1]);
+        tmem_ld_16x128b(tq2 + cD + cw, vd[h][2], vd[h][3]);
+      }
       tmem_wait_ld();
-      float lp[4], lm[4];
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        if constexpr (INF) {
-          lp[k] = __uint_as_float(vc[k]) + bo[k];
-          lm[k] = __uint_as_float(vd[k]) + bo[k];
-        } else {
-          const float C = __uint_as_float(vc[k]) + bo[k];
-          const float D = fmaf(eps, __uint_as_float(vd[k]), dbo[k]);
-          lp[k] = C + D;
-          lm[k] = C - D;
-        }
-      }
-      float mp = fmaxf(fmaxf(lp[0], lp[1]), fmaxf(lp[2], lp[3]));
-      float mm = fmaxf(fmaxf(lm[0], lm[1]), fmaxf(lm[2], lm[3]));
+      for (int h = 0; h < 2; ++h) {
 #pragma unroll
-      for (int o = 4; o < 32; o <<= 1) {
-        mp = fmaxf(mp, __shfl_xor_sync(0xffffffffu, mp, o));
-        mm = fmaxf(mm, __shfl_xor_sync(0xffffffffu, mm, o));
-      }
-      float sp = 0.f, sm_ = 0.f;
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        sp += exp_term(lp[k] - mp);
-        sm_ += exp_term(lm[k] - mm);
-      }
-#pragma unroll
-      for (int o = 4; o < 32; o <<= 1) {
-        sp += __shfl_xor_sync(0xffffffffu, sp, o);
-        sm_ += __shfl_xor_sync(0xffffffffu, sm_, o);
-      }
-      const int b = b0 + bq;
-      if (r4 == 0 && SOMA_CHECK(((p * g.Bp + b) * 2 + 1) * 4 + q4 < g.P * g.Bp * 8, a.status)) {
-        red[((p * g.Bp + b) * 2 + 0) * 4 + q4] = make_float2(mp, sp);
-        red[((p * g.Bp + b) * 2 + 1) * 4 + q4] = make_float2(mm, sm_);
-      }
-      if constexpr (INF) {
-        // the target logit of each block's sequence, into lane (e, 0, +)
-#pragma unroll
-        for (int sg = 0; sg < 2; ++sg) {
-          const int q = inf_seq(g, T.grp, sg ? col_d(p) : col_c(p), b);
-          if (q >= s.B ||
-              !SOMA_CHECK((size_t)(seq_offset(s, T.e, 0, q) + t + 1) < a.n_bytes &&
-                              (size_t)((lane_plus * s.B_mem + s.b0 + q) * (int64_t)s.T + t) <
-                                  a.n_ply,
-                          a.status))
-            continue;
-          const int y = s.bytes[seq_offset(s, T.e, 0, q) + t + 1] - vq - r4;
-          if (y >= 0 && y < 32 && (y & 7) == 0) {
-            const int k = y >> 3;
-            const float* l = sg ? lm : lp;
-            a.ply[(lane_plus * s.B_mem + s.b0 + q) * (int64_t)s.T + t] =
-                k == 0 ? l[0] : k == 1 ? l[1] : k == 2 ? l[2] : l[3];
+        for (int k = 0; k < 4; ++k) {
+          if constexpr (INF) {
+            lp[h][k] = __uint_as_float(vc[h][k]) + G.bo[k];
+            lm[h][k] = __uint_as_float(vd[h][k]) + G.bo[k];
+          } else {
+            const float C = __uint_as_float(vc[h][k]) + G.bo[k];
+            const float D = fmaf(eps, __uint_as_float(vd[h][k]), G.dbo[k]);
+            lp[h][k] = C + D;
+            lm[h][k] = C - D;
           }
         }
-      } else if (b < s.B &&
-                 SOMA_CHECK((size_t)(seq_offset(s, T.e, i, b) + t + 1) < a.n_bytes &&
-                                (size_t)(((lane_plus + 1) * s.B_mem + s.b0 + b) * (int64_t)s.T +
-                                         t) < a.n_ply,
-                            a.status)) {
-        const int y = s.bytes[seq_offset(s, T.e, i, b) + t + 1] - vq - r4;
-        // y = 8 k for the thread that holds the target row
-        if (y >= 0 && y < 32 && (y & 7) == 0) {
-          const int k = y >> 3;
-          const float vp = k == 0 ? lp[0] : k == 1 ? lp[1] : k == 2 ? lp[2] : lp[3];
-          const float vm = k == 0 ? lm[0] : k == 1 ? lm[1] : k == 2 ? lm[2] : lm[3];
-          a.ply[((lane_plus + 0) * s.B_mem + s.b0 + b) * (int64_t)s.T + t] = vp;
-          a.ply[((lane_plus + 1) * s.B_mem + s.b0 + b) * (int64_t)s.T + t] = vm;
+        mp[h] = fmaxf(fmaxf(lp[h][0], lp[h][1]), fmaxf(lp[h][2], lp[h][3]));
+        mm[h] = fmaxf(fmaxf(lm[h][0], lm[h][1]), fmaxf(lm[h][2], lm[h][3]));
+      }
+#pragma unroll
+      for (int o = 4; o < 32; o <<= 1)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          mp[h] = fmaxf(mp[h], __shfl_xor_sync(0xffffffffu, mp[h], o));
+          mm[h] = fmaxf(mm[h], __shfl_xor_sync(0xffffffffu, mm[h], o));
+        }
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        sp[h] = sm_[h] = 0.f;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          sp[h] += exp_term(lp[h][k] - mp[h]);
+          sm_[h] += exp_term(lm[h][k] - mm[h]);
+        }
+      }
+#pragma unroll
+      for (int o = 4; o < 32; o <<= 1)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          sp[h] += __shfl_xor_sync(0xffffffffu, sp[h], o);
+          sm_[h] += __shfl_xor_sync(0xffffffffu, sm_[h], o);
+        }
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int b = b0 + h * step + bq;
+        if (b >= g.Bp) continue;  // uniform over the warp's group
+        if (r4 == 0 && SOMA_CHECK(((p * g.Bp + b) * 2 + 1) * 4 + q4 < g.P * g.Bp * 8, a.status)) {
+          red[((p * g.Bp + b) * 2 + 0) * 4 + q4] = make_float2(mp[h], sp[h]);
+          red[((p * g.Bp + b) * 2 + 1) * 4 + q4] = make_float2(mm[h], sm_[h]);
+        }
+        if constexpr (INF) {
+          // the target logit of each block's sequence, into lane (e, 0, +)
+#pragma unroll
+          for (int sg = 0; sg < 2; ++sg) {
+            const int j = 2 * (j0 + h) + sg;
+            const int q = inf_seq(g, T.grp, sg ? col_d(p) : col_c(p), b);
+            const int y = (int)((G.tgt[j >> 2] >> (8 * (j & 3))) & 255u) - vq - r4;
+            if (q < s.B && y >= 0 && y < 32 && (y & 7) == 0 &&
+                SOMA_CHECK((size_t)((lane_plus * s.B_mem + s.b0 + q) * (int64_t)s.T + t) < a.n_ply,
+                           a.status)) {
+              const int k = y >> 3;
+              const float* l = sg ? lm[h] : lp[h];
+              a.ply[(lane_plus * s.B_mem + s.b0 + q) * (int64_t)s.T + t] =
+                  k == 0 ? l[0] : k == 1 ? l[1] : k == 2 ? l[2] : l[3];
+            }
+          }
+        } else {
+          const int j = j0 + h;
+          const int y = (int)((G.tgt[j >> 2] >> (8 * (j & 3))) & 255u) - vq - r4;
+          // y = 8 k for the thread that holds the target row
+          if (b < s.B && y >= 0 && y < 32 && (y & 7) == 0 &&
+              SOMA_CHECK((size_t)(((lane_plus + 1) * s.B_mem + s.b0 + b) * (int64_t)s.T + t) <
+                             a.n_ply,
+                         a.status)) {
+            const int k = y >> 3;
+            const float vp = k == 0 ? lp[h][0] : k == 1 ? lp[h][1] : k == 2 ? lp[h][2] : lp[h][3];
+            const float vm = k == 0 ? lm[h][0] : k == 1 ? lm[h][1] : k == 2 ? lm[h][2] : lm[h][3];
+            a.ply[((lane_plus + 0) * s.B_mem + s.b0 + b) * (int64_t)s.T + t] = vp;
+            a.ply[((lane_plus + 1) * s.B_mem + s.b0 + b) * (int64_t)s.T + t] = vm;
+          }
         }
       }
     }
   }
   // all epilogue warps: partials of this task are in `red`
   if (!epi_rendezvous(red_bar, red_use, abort, a.status)) return false;
-  const int et = threadIdx.x - kEpiWarp0 * 32;
+  const int et = ew * 32 + lane;
   const int n_red = T.p_valid * g.Bp * 2;
-  for (int idx = et; idx < n_red; idx += kEpiWarps * 32) {
+  for (int idx = et; idx < n_red; idx += EPI * 32) {
     const int sgn = idx & 1;
     const int pb = idx >> 1;
     const int pp = pb / g.Bp, b = pb % g.Bp;
@@ -912,11 +992,13 @@ __device__ __forceinline__ uint8_t* align1024(uint8_t* p) {
 }
 
 // grid: one persistent CTA per SM at most (all resident: the launch is
-// cooperative), kThreads threads.  The CTAs share the tasks of phases
+// cooperative), Warps<INF, EPI>::threads threads.  The CTAs share the tasks of phases
 // 0 .. T through the task counter.
 // SPARSE: sparse probes; INF: the unperturbed layout (eps = 0, one sign).
-template <bool SPARSE, bool INF>
-__global__ void __launch_bounds__(kThreads, 1) tc_persistent_kernel(const TcArgs a) {
+template <bool SPARSE, bool INF, int EPI>
+__global__ void __launch_bounds__((Warps<INF, EPI>::threads), 1)
+tc_persistent_kernel(const TcArgs a) {
+  constexpr int kEpi = EPI, kFirstEpi = Warps<INF, EPI>::epi0;
   extern __shared__ uint8_t dyn_smem[];
   const TcGeom& g = a.g;
   const Sweep& s = a.sw;
@@ -934,22 +1016,22 @@ __global__ void __launch_bounds__(kThreads, 1) tc_persistent_kernel(const TcArgs
     for (int q = 0; q < kStages; ++q) {
       // the loader's arrival with the copies' bytes and, when probes are
       // generated, one arrival per Z warp
-      mbar_init(&ctl->full[q], do_z ? 1 + kZWarps : 1);
+      mbar_init(&ctl->full[q], !INF && do_z ? 1 + kZWarps : 1);
       mbar_init(&ctl->slot_free[q], 1);
     }
     for (int q = 0; q < kZSlots; ++q) mbar_init(&ctl->z_free[q], 1);
     for (int q = 0; q < 2; ++q) {
       mbar_init(&ctl->acc_full[q], 1);
-      mbar_init(&ctl->acc_empty[q], kEpiWarps);
+      mbar_init(&ctl->acc_empty[q], kEpi);
     }
-    mbar_init(&ctl->red_bar, kEpiWarps);
+    mbar_init(&ctl->red_bar, kEpi);
     mbar_init(&ctl->mma_done, 1);
     for (int q = 0; q < kTaskSlots; ++q) {
       mbar_init(&ctl->task_full[q], 1);
       // the loader, the MMA issuer, the Z warps (when probes are
       // generated), the epilogue warps and the releaser read every task
-      mbar_init(&ctl->task_empty[q], 3 + (do_z ? kZWarps : 0) + kEpiWarps);
-      mbar_init(&ctl->task_done[q], kEpiWarps);
+      mbar_init(&ctl->task_empty[q], 3 + (!INF && do_z ? kZWarps : 0) + kEpi);
+      mbar_init(&ctl->task_done[q], kEpi);
     }
     mbar_fence_init();
   }
@@ -1139,12 +1221,12 @@ __global__ void __launch_bounds__(kThreads, 1) tc_persistent_kernel(const TcArgs
         break;
       if (lane == 0) {
         __threadfence();
-        atomicAdd(T.head ? a.hd + c : a.prod + c, kEpiWarps);
+        atomicAdd(T.head ? a.hd + c : a.prod + c, 1);
         mbar_arrive(&ctl->task_empty[sl]);
       }
       __syncwarp();
     }
-  } else if (warp >= kZWarp0 && warp < kEpiWarp0) {
+  } else if (!INF && warp >= kZWarp0 && warp < kFirstEpi) {
     // --------------------------------------------------------- Z generators
     // Thread (probe gtid / 128, row gtid % 128 = TMEM lane).  The raw probe
     // words of a stage come from the table zbits_block wrote before the
@@ -1240,7 +1322,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_persistent_kernel(const TcArgs
         }
       }
     }
-  } else if (warp >= kEpiWarp0) {
+  } else if (warp >= kFirstEpi) {
     // --------------------------------------------------------------- epilogue
     // A gate task of phase t overwrites what phase t - 1 read (op[(t + 1) %
     // 2]) and reads the cell states that phase t - 1 wrote, possibly in
@@ -1248,7 +1330,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_persistent_kernel(const TcArgs
     // group's counters of phase t - 1.  After each task it
     // arrives on the task's done barrier, and the releaser publishes the
     // task on the group's counter.
-    const int ew = warp - kEpiWarp0;
+    const int ew = warp - kFirstEpi;
     const int q4 = warp & 3;
     int k = 0;
     uint32_t red_use = 0;
@@ -1262,22 +1344,27 @@ __global__ void __launch_bounds__(kThreads, 1) tc_persistent_kernel(const TcArgs
       {
         const int buf = k & 1;
         const size_t c = (size_t)T.e * g.G + T.grp;
-        GatePre G;
-        if (!SOMA_CHECK(c < (size_t)g.n_experts * g.G, status) ||
-            !wait_or_abort(&ctl->acc_full[buf], (uint32_t)(k >> 1) & 1u, abort, status)) {
+        const uint32_t tacc = tmem + (uint32_t)buf * kAccCols;
+        if (!SOMA_CHECK(c < (size_t)g.n_experts * g.G, status)) {
           alive = false;
           break;
         }
-        if (!T.head) gate_prepare<INF>(a, ph, T, q4, ew >> 2, G);
-        tc_fence_after();
-        const uint32_t tacc = tmem + (uint32_t)buf * kAccCols;
+        // what does not depend on the accumulator is loaded under its MMAs
         if (T.head) {
-          if (!head_epilogue<INF>(a, ph, T, tacc, q4, ew, red, &ctl->red_bar, &red_use, abort)) {
-            alive = false;
-            break;
-          }
+          HeadPre G;
+          head_prepare<INF, EPI>(a, ph, T, q4, ew, G);
+          alive = wait_or_abort(&ctl->acc_full[buf], (uint32_t)(k >> 1) & 1u, abort, status);
+          if (!__all_sync(0xffffffffu, alive)) break;
+          tc_fence_after();
+          alive = head_epilogue<INF, EPI>(a, ph, T, tacc, q4, ew, G, red, &ctl->red_bar, &red_use, abort);
+          if (!__all_sync(0xffffffffu, alive)) break;
         } else {
-          gate_finish<INF>(a, ph, T, tacc, q4, G);
+          GatePre<EPI> G;
+          gate_prepare<INF, EPI>(a, ph, T, q4, ew, G);
+          alive = wait_or_abort(&ctl->acc_full[buf], (uint32_t)(k >> 1) & 1u, abort, status);
+          if (!__all_sync(0xffffffffu, alive)) break;
+          tc_fence_after();
+          gate_finish<INF, EPI>(a, ph, T, tacc, q4, G);
         }
         tc_fence_before();
         __syncwarp();
@@ -1665,6 +1752,18 @@ debug_tc_gemm_kernel(const __half* A, const __half* B, float* D, int N, int K, i
   if (tid < 32) tmem_dealloc(tmem, 512);
 }
 
+// Epilogue warps of a perturbed sweep.  With few stages along K a task's MMAs
+// take less time than its epilogue on 8 warps, and 16 are worth the registers
+// (72 a thread instead of 96); with many stages, or more generator work per stage
+// (sparse probes), the extra warps only compete for issue slots, and with fewer
+// tasks than SMs nothing waits for an epilogue.  Measured, time with 8 over time
+// with 16 (8 experts, 64 probes, 32 sequences), dense: 1.28 at S = 3 stages, 1.22
+// at 5, 1.15 at 7, 1.05 at 8, 0.97 at 9, 0.96 at 16; sparse: 1.25, 1.19, 1.01,
+// 0.96, 0.91, 0.91; 16 to 60 tasks on 152 SMs: 0.97 to 1.00.
+int epi_warps_for(const TcGeom& g, bool sparse, int tasks) {
+  return tasks > sm_count() && g.S <= (sparse ? 7 : 8) ? 16 : 8;
+}
+
 size_t kernel_smem_bytes(const TcGeom& g) {
   // ring slots, the control block (1 KB), the head's reduction buffer
   // [P][Bp][2][4] float2 and alignment slack
@@ -1752,8 +1851,15 @@ TcSizes tc_sizes(const TcGeom& g) {
 cudaError_t launch_forward_tc(const Sweep& s, const TcGeom& g, const TcBuffers& tb, int* status,
                               cudaStream_t stream) {
   const size_t smem = kernel_smem_bytes(g);
-  auto kernel = g.inf ? tc_persistent_kernel<false, true>
-                      : s.sparse ? tc_persistent_kernel<true, false> : tc_persistent_kernel<false, false>;
+  const int epi = g.inf ? kInfEpi : epi_warps_for(g, s.sparse != 0, g.n_experts * (g.MT + 2) * g.G);
+  auto kernel = g.inf ? tc_persistent_kernel<false, true, kInfEpi>
+                : epi == 16
+                    ? (s.sparse ? tc_persistent_kernel<true, false, 16>
+                                : tc_persistent_kernel<false, false, 16>)
+                    : (s.sparse ? tc_persistent_kernel<true, false, 8>
+                                : tc_persistent_kernel<false, false, 8>);
+  const int threads = g.inf ? Warps<true, kInfEpi>::threads
+                            : epi == 16 ? Warps<false, 16>::threads : Warps<false, 8>::threads;
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem);
   if (e != cudaSuccess) return e;
@@ -1826,7 +1932,7 @@ cudaError_t launch_forward_tc(const Sweep& s, const TcGeom& g, const TcBuffers& 
   // every phase of the sweep in one cooperative launch: its CTAs wait on
   // each other's phase counters, so all of them must be resident together
   int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kThreads, smem);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem);
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorLaunchOutOfResources;
   const int sms = sm_count();
@@ -1834,7 +1940,7 @@ cudaError_t launch_forward_tc(const Sweep& s, const TcGeom& g, const TcBuffers& 
   const int ctas = tasks < sms ? tasks : sms;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)ctas);
-  cfg.blockDim = dim3(kThreads);
+  cfg.blockDim = dim3((unsigned)threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
   cudaLaunchAttribute attr[1];

@@ -126,6 +126,16 @@ __host__ __device__ __forceinline__ ProbeBits probe_bits(const ProbeKey& k, int6
   return b;
 }
 
+// The same for parameter p alone, in bit 0: one Philox block per stream.
+__host__ __device__ __forceinline__ ProbeBits probe_bit(const ProbeKey& k, int64_t p, bool sparse) {
+  const uint32_t w = (uint32_t)(p >> 5);
+  const int bit = raw_bit((int)(p & 31));
+  ProbeBits b;
+  b.neg = (probe_raw_word(k, w) >> bit) & 1u;
+  b.act = sparse ? (probe_raw_word(activity_key(k), w) >> bit) & 1u : 1u;
+  return b;
+}
+
 // w + s*eps*z for a z bit: the perturbed parameter in fp32.
 __host__ __device__ __forceinline__ float perturb(float w, uint32_t bit, float se) {
   return w + (bit ? -se : se);
