@@ -60,7 +60,11 @@ using namespace tc;
 
 namespace {
 
-constexpr int kStages = 5;       // ring slots of the shared-memory operands (W and operand tiles)
+// Ring slots of the shared-memory operands (W and operand tiles): 40 KB each,
+// 32 KB in the unperturbed layout, which copies only the 128 operand rows its
+// W product reads.
+constexpr int kMaxStages = 6;
+__host__ __device__ constexpr int ring_stages(bool inf) { return inf ? kMaxStages : 5; }
 constexpr int kZSlots = 4;       // ring slots of the TMEM probe tiles (TMEM holds no more)
 // Each stage's two copies (W tile, operand tile) are one 2-lane bulk-copy
 // instruction of one loader warp.  The copies of one warp complete one after
@@ -134,14 +138,18 @@ __device__ __forceinline__ int cst_lanes_of(const TcGeom& g) {
 
 // Shared-memory carve-up of one ring slot.
 struct StageLayout {
-  uint32_t a_off, b_off, bytes;
+  uint32_t a_off, b_off, b_src, b_bytes, bytes;
 };
 
 __host__ __device__ inline StageLayout stage_layout(const TcGeom& g) {
   StageLayout L;
   L.a_off = 0;
   L.b_off = kTileA;
-  L.bytes = (L.b_off + g.tileB + 1023u) & ~1023u;
+  // the operand rows a stage holds: all of the group tile, or (unperturbed) the
+  // four sequence blocks
+  L.b_src = g.inf ? (uint32_t)(g.Bp / 8) * kSbo : 0u;
+  L.b_bytes = g.inf ? (uint32_t)(4 * g.Bp / 8) * kSbo : g.tileB;
+  L.bytes = (L.b_off + L.b_bytes + 1023u) & ~1023u;
   return L;
 }
 
@@ -286,8 +294,8 @@ struct Task {
 };
 
 struct Ctl {
-  uint64_t full[kStages];
-  uint64_t slot_free[kStages];
+  uint64_t full[kMaxStages];
+  uint64_t slot_free[kMaxStages];
   uint64_t z_free[kZSlots];        // the MMAs reading a probe-tile slot are done
   uint64_t acc_full[2];
   uint64_t acc_empty[2];
@@ -323,10 +331,11 @@ __device__ __forceinline__ bool wait_or_abort(uint64_t* bar, uint32_t parity, vo
 
 // Ring position of the next stage: shared-memory slot q and the parity of
 // its phase, probe-tile slot zq.
+template <int STAGES>
 struct RingPos {
   uint32_t q, ph, zq;
   __device__ __forceinline__ void next() {
-    if (++q == kStages) {
+    if (++q == STAGES) {
       q = 0;
       ph ^= 1u;
     }
@@ -338,9 +347,9 @@ struct RingPos {
 // copies and the probe tiles (one barrier), issue, and release the slot
 // with a commit.
 // The probe count NP is fixed per task, so the loop carries no dispatch.
-template <int NP>
+template <int NP, int STAGES>
 __device__ __forceinline__ bool mma_task(uint64_t* full, uint64_t* slot_free, uint64_t* z_free,
-                                         RingPos& rp, int nst, uint32_t d, uint32_t tmem,
+                                         RingPos<STAGES>& rp, int nst, uint32_t d, uint32_t tmem,
                                          uint32_t a_lo0, uint32_t b_lo0, uint32_t slot_step,
                                          uint32_t hi, uint32_t w_row, uint32_t z1_row,
                                          uint32_t idesc_w, uint32_t idesc_z, uint32_t dz1,
@@ -356,7 +365,7 @@ __device__ __forceinline__ bool mma_task(uint64_t* full, uint64_t* slot_free, ui
     // allocations
     if (!SOMA_CHECK((d & 0xFFFFu) + dz1 + (NP >= 2 ? dz1 : 0) <= 2 * kAccCols &&
                         kZCol0 + 64u * rp.zq + 32u * (NP > 0 ? NP : 1) <= kTmemCols &&
-                        rp.q < (uint32_t)kStages && rp.zq < (uint32_t)kZSlots,
+                        rp.q < (uint32_t)STAGES && rp.zq < (uint32_t)kZSlots,
                     status))
       return false;
     const uint32_t so = rp.q * slot_step;
@@ -998,7 +1007,7 @@ __device__ __forceinline__ uint8_t* align1024(uint8_t* p) {
 template <bool SPARSE, bool INF, int EPI>
 __global__ void __launch_bounds__((Warps<INF, EPI>::threads), 1)
 tc_persistent_kernel(const TcArgs a) {
-  constexpr int kEpi = EPI, kFirstEpi = Warps<INF, EPI>::epi0;
+  constexpr int kEpi = EPI, kFirstEpi = Warps<INF, EPI>::epi0, kStages = ring_stages(INF);
   extern __shared__ uint8_t dyn_smem[];
   const TcGeom& g = a.g;
   const Sweep& s = a.sw;
@@ -1108,14 +1117,14 @@ tc_persistent_kernel(const TcArgs a) {
             break;
           }
           uint8_t* slot = smem + q * SL.bytes;
-          if (lane == 0) mbar_arrive_expect_tx(&ctl->full[q], kTileA + g.tileB);
+          if (lane == 0) mbar_arrive_expect_tx(&ctl->full[q], kTileA + SL.b_bytes);
           __syncwarp();
           if (lane < 2) {
             uint8_t* dst = lane == 0 ? slot + SL.a_off : slot + SL.b_off;
             const bool xs = !T.head && st < g.Sx;  // an embedding-part stage
             const uint8_t* src = lane == 0 ? T.a + (size_t)st * kTileA
-                                           : (xs ? T.bx : T.b) + (size_t)st * g.G * g.tileB;
-            const uint32_t nb = lane == 0 ? kTileA : g.tileB;
+                                           : (xs ? T.bx : T.b) + (size_t)st * g.G * g.tileB + SL.b_src;
+            const uint32_t nb = lane == 0 ? kTileA : SL.b_bytes;
             const uint8_t* gbase =
                 lane == 1 ? (xs ? a.xall : ph.op_in) : (T.head ? a.wo16 : a.w16);
             const size_t gsize =
@@ -1159,10 +1168,11 @@ tc_persistent_kernel(const TcArgs a) {
       const uint32_t slot_step = SL.bytes >> 4;
       const uint32_t a_lo0 = lo0 + (SL.a_off >> 4), b_lo0 = lo0 + (SL.b_off >> 4);
       const uint32_t grp_step = kSbo >> 4;                     // 8 operand rows
-      const uint32_t w_row = (uint32_t)(g.Bp / 8) * grp_step;  // the W window starts at row Bp
+      // the W window starts at row Bp of the group tile
+      const uint32_t w_row = (uint32_t)(g.Bp / 8) * grp_step - (SL.b_src >> 4);
       const uint32_t z1_row = (uint32_t)(4 * g.Bp / 8) * grp_step;
       const uint32_t dz1 = (uint32_t)(2 * g.Bp);
-      RingPos rp = {0u, 0u, 0u};
+      RingPos<kStages> rp = {0u, 0u, 0u};
       uint32_t kt = 0;
       for (int k = 0;; ++k) {
         int t;
@@ -1178,13 +1188,13 @@ tc_persistent_kernel(const TcArgs a) {
         const int np = do_z ? T.p_valid : 0;
         bool ok;
         if (np == 2)
-          ok = mma_task<2>(ctl->full, ctl->slot_free, ctl->z_free, rp, T.nst, d, tmem, a_lo0, b_lo0,
+          ok = mma_task<2, kStages>(ctl->full, ctl->slot_free, ctl->z_free, rp, T.nst, d, tmem, a_lo0, b_lo0,
                            slot_step, hi, w_row, z1_row, idesc_w, idesc_z, dz1, abort, status);
         else if (np == 1)
-          ok = mma_task<1>(ctl->full, ctl->slot_free, ctl->z_free, rp, T.nst, d, tmem, a_lo0, b_lo0,
+          ok = mma_task<1, kStages>(ctl->full, ctl->slot_free, ctl->z_free, rp, T.nst, d, tmem, a_lo0, b_lo0,
                            slot_step, hi, w_row, z1_row, idesc_w, idesc_z, dz1, abort, status);
         else
-          ok = mma_task<0>(ctl->full, ctl->slot_free, ctl->z_free, rp, T.nst, d, tmem, a_lo0, b_lo0,
+          ok = mma_task<0, kStages>(ctl->full, ctl->slot_free, ctl->z_free, rp, T.nst, d, tmem, a_lo0, b_lo0,
                            slot_step, hi, w_row, z1_row, idesc_w, idesc_z, dz1, abort, status);
         if (!ok) break;
         if (elect_one()) mma_commit(&ctl->acc_full[buf]);
@@ -1768,7 +1778,7 @@ size_t kernel_smem_bytes(const TcGeom& g) {
   // ring slots, the control block (1 KB), the head's reduction buffer
   // [P][Bp][2][4] float2 and alignment slack
   const size_t red = (size_t)g.P * g.Bp * 2 * 4 * sizeof(float2);
-  return (size_t)kStages * stage_layout(g).bytes + 1024 + red + 1024;
+  return (size_t)ring_stages(g.inf != 0) * stage_layout(g).bytes + 1024 + red + 1024;
 }
 
 }  // namespace
