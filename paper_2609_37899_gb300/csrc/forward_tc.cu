@@ -60,11 +60,14 @@ using namespace tc;
 
 namespace {
 
-// Ring slots of the shared-memory operands (W and operand tiles): 40 KB each,
-// 32 KB in the unperturbed layout, which copies only the 128 operand rows its
-// W product reads.
+constexpr int kKt = 64;                     // K per stage (fp16 elements)
+constexpr uint32_t kTileA = 128 * kKt * 2;  // one 128-row A tile per stage
+// Ring slots of the shared-memory operands (W and operand tiles): five of 40
+// KB; in the unperturbed layout four of up to 48 KB, or six of up to 32.
 constexpr int kMaxStages = 6;
-__host__ __device__ constexpr int ring_stages(bool inf) { return inf ? kMaxStages : 5; }
+__host__ __device__ inline int ring_stages(const TcGeom& g) {
+  return !g.inf ? 5 : g.tileB <= kTileA ? 6 : 4;
+}
 constexpr int kZSlots = 4;       // ring slots of the TMEM probe tiles (TMEM holds no more)
 // Each stage's two copies (W tile, operand tile) are one 2-lane bulk-copy
 // instruction of one loader warp.  The copies of one warp complete one after
@@ -86,11 +89,11 @@ struct Warps {
 };
 static_assert(kZWarp0 % 4 == 0 && kZWarps % 4 == 0, "warp w reads TMEM lane quarter w % 4");
 constexpr int kTaskSlots = 4;               // tasks a CTA's fetcher publishes ahead of the others
-constexpr int kKt = 64;                     // K per stage (fp16 elements)
-constexpr uint32_t kTileA = 128 * kKt * 2;  // one 128-row A tile per stage
 constexpr uint32_t kSbo = kKt * 16;         // bytes between 8-row groups
 constexpr uint32_t kLbo = 128;              // bytes between core matrices along K
 constexpr uint32_t kAccCols = 128;          // one accumulator buffer: 2 Bp P <= 128 columns
+// (unperturbed: 8 blocks of 32 sequences, and no probe tiles beside the two buffers)
+__host__ __device__ constexpr uint32_t acc_cols(bool inf) { return inf ? 2 * kAccCols : kAccCols; }
 constexpr uint32_t kZCol0 = 2 * kAccCols;   // probe tiles: slot q at kZCol0 + 64 q (+ 32 p)
 constexpr uint32_t kTmemCols = 512;
 static_assert(kZCol0 + kZSlots * 64 <= kTmemCols, "probe tiles fit tensor memory");
@@ -118,37 +121,43 @@ __host__ __device__ __forceinline__ int row_e2(int p) { return p == 0 ? 0 : 5; }
 __host__ __device__ __forceinline__ int col_c(int p) { return row_mean(p) - 1; }
 __host__ __device__ __forceinline__ int col_d(int p) { return row_dhat(p) - 1; }
 
-// The unperturbed layout: accumulator column block j (and operand row block
-// j + 1) holds sequences (4 grp + j) Bp .. + Bp - 1 of the expert's batch.
-// "Probe" p of a group then stands for the two blocks col_c(p) (its + lane)
-// and col_d(p) (its - lane), and its cell states sit where a probe's two
-// signs sit in the perturbed layout.
+// The unperturbed layout: accumulator column block j and operand row block j
+// (up to 8 per group) hold sequences (8 grp + j) Bp .. + Bp - 1 of the expert's
+// batch.  "Probe" p of a group then stands for the blocks 2p (its + lane) and
+// 2p + 1 (its - lane), and its cell states sit where a probe's two signs sit
+// in the perturbed layout.
 __host__ __device__ __forceinline__ int inf_seq(const TcGeom& g, int grp, int blk, int b) {
-  return (4 * grp + blk) * g.Bp + b;
+  return (g.blocks * grp + blk) * g.Bp + b;
 }
+// Sequence blocks of a group.
+__host__ __device__ __forceinline__ int inf_blocks(const TcGeom& g, int grp) {
+  const int left = (g.B + g.Bp - 1) / g.Bp - g.blocks * grp;
+  return left < g.blocks ? left : g.blocks;
+}
+template <bool INF>
+__host__ __device__ __forceinline__ int blk_c(int p) { return INF ? 2 * p : col_c(p); }
+template <bool INF>
+__host__ __device__ __forceinline__ int blk_d(int p) { return INF ? 2 * p + 1 : col_d(p); }
 
 // Probe slots of the cell-state buffer per expert.
 __host__ __device__ __forceinline__ int cst_lanes(const TcGeom& g) {
-  return g.inf ? 2 * g.G : g.n_pert;
+  return g.inf ? ((g.B + g.Bp - 1) / g.Bp + 1) / 2 : g.n_pert;
 }
 template <bool INF>
 __device__ __forceinline__ int cst_lanes_of(const TcGeom& g) {
-  return INF ? 2 * g.G : g.n_pert;
+  return INF ? ((g.B + g.Bp - 1) / g.Bp + 1) / 2 : g.n_pert;
 }
 
 // Shared-memory carve-up of one ring slot.
 struct StageLayout {
-  uint32_t a_off, b_off, b_src, b_bytes, bytes;
+  uint32_t a_off, b_off, b_bytes, bytes;
 };
 
 __host__ __device__ inline StageLayout stage_layout(const TcGeom& g) {
   StageLayout L;
   L.a_off = 0;
   L.b_off = kTileA;
-  // the operand rows a stage holds: all of the group tile, or (unperturbed) the
-  // four sequence blocks
-  L.b_src = g.inf ? (uint32_t)(g.Bp / 8) * kSbo : 0u;
-  L.b_bytes = g.inf ? (uint32_t)(4 * g.Bp / 8) * kSbo : g.tileB;
+  L.b_bytes = g.tileB;
   L.bytes = (L.b_off + L.b_bytes + 1023u) & ~1023u;
   return L;
 }
@@ -363,7 +372,7 @@ __device__ __forceinline__ bool mma_task(uint64_t* full, uint64_t* slot_free, ui
     // the accumulator block, the probe tiles of the slot and the operand
     // windows (rows of 128 bytes per 8-row group step) stay inside their
     // allocations
-    if (!SOMA_CHECK((d & 0xFFFFu) + dz1 + (NP >= 2 ? dz1 : 0) <= 2 * kAccCols &&
+    if (!SOMA_CHECK((NP == 0 || (d & 0xFFFFu) + dz1 + (NP >= 2 ? dz1 : 0) <= 2 * kAccCols) &&
                         kZCol0 + 64u * rp.zq + 32u * (NP > 0 ? NP : 1) <= kTmemCols &&
                         rp.q < (uint32_t)STAGES && rp.zq < (uint32_t)kZSlots,
                     status))
@@ -529,7 +538,7 @@ __device__ __forceinline__ Task make_task(const TcArgs& a, const Phase& ph, int 
   T.m = T.head ? w : w - hb;
   T.grp = block % g.G;
   T.e = block / g.G;
-  T.p_valid = INF ? g.P : min(g.P, a.sw.n_pert - T.grp * g.P);
+  T.p_valid = INF ? (inf_blocks(g, T.grp) + 1) / 2 : min(g.P, a.sw.n_pert - T.grp * g.P);
   if (T.head) {
     T.nst = g.Sh;
     T.a = a.wo16 + (((size_t)T.e * 2 + T.m) * g.Sh) * kTileA;
@@ -571,16 +580,18 @@ __host__ __device__ __forceinline__ size_t zbits_row(const TcGeom& g, int e, int
 }
 
 // The share of an epilogue warp: TMEM lane quarter w % 4 of one probe p, and of
-// its sequence chunks those c with c % parts == part.  With P = 2 the warp groups
-// eg = ew / 4 alternate between the probes, with P = 1 all run probe 0.
+// its sequence chunks those c with c % parts == part.  The warp groups eg = ew / 4
+// split over the probes (unperturbed: the pairs of blocks), then over each
+// one's chunks.
 struct EpiShare {
   int p, part, parts;
 };
-template <int EPI>
-__device__ __forceinline__ EpiShare epi_share(const TcGeom& g, int ew) {
+template <bool INF, int EPI>
+__device__ __forceinline__ EpiShare epi_share(const TcGeom& g, int p_valid, int ew) {
   constexpr int groups = EPI / 4;
-  const int eg = ew >> 2;
-  if (g.P == 2) return {eg & 1, eg >> 1, groups / 2};
+  const int eg = ew >> 2, over = INF ? p_valid : g.P;
+  if (INF && over > 2) return {eg, 0, 1};
+  if (over == 2) return {eg & 1, eg >> 1, groups / 2};
   return {0, eg, groups};
 }
 
@@ -596,10 +607,10 @@ __device__ __forceinline__ EpiShare epi_share(const TcGeom& g, int ew) {
 // gate_prepare runs before the accumulator is ready: it loads the bias, its
 // probe signs and the previous cell states, so that their latency overlaps
 // the task's MMAs.
-// Chunks of one warp: Bp <= 32 with P = 2, Bp <= 64 with P = 1.
-template <int EPI>
+// Chunks of one warp: Bp <= 32 with P = 2 (or unperturbed), Bp <= 64 with P = 1.
+template <bool INF, int EPI>
 struct GatePre {
-  static constexpr int chunks = 32 / EPI;
+  static constexpr int chunks = INF ? 4 : 32 / EPI;
   float bias[4], dbias[4];
   float2 cprev[chunks][2];
   int p, c0, cstep;
@@ -608,19 +619,20 @@ struct GatePre {
 
 template <bool INF, int EPI>
 __device__ __forceinline__ void gate_prepare(const TcArgs& a, const Phase& ph, const Task& T,
-                                             int q4, int ew, GatePre<EPI>& G) {
+                                             int q4, int ew, GatePre<INF, EPI>& G) {
   const TcGeom& g = a.g;
   const Sweep& s = a.sw;
   const Layout& L = s.lay;
   const int lane = threadIdx.x & 31;
   const int H = g.H;
-  const EpiShare sh = epi_share<EPI>(g, ew);
+  const EpiShare sh = epi_share<INF, EPI>(g, T.p_valid, ew);
   G.p = sh.p;
   G.c0 = sh.part;
   G.cstep = sh.parts;
   G.on = G.p < T.p_valid;
   if (!G.on) return;
   const int i = T.grp * g.P + G.p;
+  const int ci = INF ? g.blocks / 2 * T.grp + G.p : i;
   const ProbeKey pk = make_probe_key(s.seed, s.step, (uint32_t)T.e, (uint32_t)i);
   const float eps = s.eps;
   const float* th = s.params + (int64_t)T.e * L.P;
@@ -628,10 +640,10 @@ __device__ __forceinline__ void gate_prepare(const TcArgs& a, const Phase& ph, c
   const int u8 = lane >> 2, bq = lane & 3;
   const int U = 32 * T.m + 8 * q4 + u8;
   const float2* cell = reinterpret_cast<const float2*>(a.cst) +
-                       (((int64_t)T.e * cst_lanes_of<INF>(g) + i) * g.Hp + U) * (int64_t)g.Bp;
+                       (((int64_t)T.e * cst_lanes_of<INF>(g) + ci) * g.Hp + U) * (int64_t)g.Bp;
   const bool load = U < H && ph.t_gate > 0;
 #pragma unroll
-  for (int j = 0; j < GatePre<EPI>::chunks; ++j) {
+  for (int j = 0; j < GatePre<INF, EPI>::chunks; ++j) {
     const int b0 = 8 * (G.c0 + j * G.cstep);
     G.cprev[j][0] = G.cprev[j][1] = make_float2(0.f, 0.f);
     if (load && b0 < g.Bp &&
@@ -664,7 +676,7 @@ __device__ __forceinline__ void gate_prepare(const TcArgs& a, const Phase& ph, c
 
 template <bool INF, int EPI>
 __device__ void gate_finish(const TcArgs& a, const Phase& ph, const Task& T, uint32_t tacc,
-                            int q4, const GatePre<EPI>& G) {
+                            int q4, const GatePre<INF, EPI>& G) {
   if (!G.on) return;
   const TcGeom& g = a.g;
   const Sweep& s = a.sw;
@@ -681,20 +693,21 @@ __device__ void gate_finish(const TcArgs& a, const Phase& ph, const Task& T, uin
   uint8_t* out_tile =
       ph.op_out + (((size_t)T.e * g.S + g.Sx + 32 * T.m / kKt) * g.G + T.grp) * g.tileB;
   const int kk = 32 * T.m % kKt + 8 * q4 + u8;
-  const int i = T.grp * g.P + p;
+  const int ci = (INF ? g.blocks / 2 : g.P) * T.grp + p;
   float2* cell = reinterpret_cast<float2*>(a.cst) +
-                 (((int64_t)T.e * cst_lanes_of<INF>(g) + i) * g.Hp + U) * (int64_t)g.Bp;
+                 (((int64_t)T.e * cst_lanes_of<INF>(g) + ci) * g.Hp + U) * (int64_t)g.Bp;
   const uint32_t tq = tacc + ((uint32_t)(32 * q4) << 16);  // gates 0, 1
   const uint32_t tq2 = tq + (16u << 16);                    // gates 2, 3
-  const uint32_t cC = (uint32_t)(col_c(p) * g.Bp), cD = (uint32_t)(col_d(p) * g.Bp);
-  const int rM = row_mean(p) * g.Bp, rD = row_dhat(p) * g.Bp, rE = row_e2(p) * g.Bp;
+  const uint32_t cC = (uint32_t)(blk_c<INF>(p) * g.Bp), cD = (uint32_t)(blk_d<INF>(p) * g.Bp);
+  const int rM = (INF ? 2 * p : row_mean(p)) * g.Bp, rD = (INF ? 2 * p + 1 : row_dhat(p)) * g.Bp,
+            rE = INF ? 0 : row_e2(p) * g.Bp;
 #pragma unroll
-  for (int j = 0; j < GatePre<EPI>::chunks; ++j) {
+  for (int j = 0; j < GatePre<INF, EPI>::chunks; ++j) {
     const int b0 = 8 * (G.c0 + j * G.cstep);
     if (b0 >= g.Bp) break;
     // [seq half][gate]: C (W vbar + eps^2 Z dhat) and D (W dhat + Z vbar)
     uint32_t vc[2][4], vd[2][4];
-    if (!SOMA_CHECK(cC + b0 + 8 <= kAccCols && cD + b0 + 8 <= kAccCols, a.status)) break;
+    if (!SOMA_CHECK(cC + b0 + 8 <= acc_cols(INF) && cD + b0 + 8 <= acc_cols(INF), a.status)) break;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const uint32_t cw = (uint32_t)(b0 + 4 * h);
@@ -744,16 +757,16 @@ __device__ void gate_finish(const TcArgs& a, const Phase& ph, const Task& T, uin
       const size_t tile_off = (size_t)(out_tile - ph.op_out);
       if (unit_ok &&
           SOMA_CHECK((size_t)(cell - reinterpret_cast<float2*>(a.cst) + b + 1) * 2 <= a.n_cst &&
-                         tile_off + g.tileB <= a.n_op && rE + b < g.rowsB && rD + b < g.rowsB &&
-                         rM + b < g.rowsB && kk < kKt,
+                         tile_off + g.tileB <= a.n_op && rE + b < g.rowsB &&
+                         (INF || (rD + b < g.rowsB && rM + b < g.rowsB)) && kk < kKt,
                      a.status)) {
         cell[b] = make_float2(cp, cm);
         if constexpr (INF) {
           // h of the two blocks into their own rows (the W product's rows)
-          if (inf_seq(g, T.grp, col_c(p), b) < s.B)
+          if (inf_seq(g, T.grp, 2 * p, b) < s.B)
             *reinterpret_cast<__half*>(out_tile + kmajor_offset(rM + b, kk, kKt)) =
                 __float2half_rn(actp[3] * tp);
-          if (inf_seq(g, T.grp, col_d(p), b) < s.B)
+          if (inf_seq(g, T.grp, 2 * p + 1, b) < s.B)
             *reinterpret_cast<__half*>(out_tile + kmajor_offset(rD + b, kk, kKt)) =
                 __float2half_rn(actm[3] * tm);
         } else if (b < s.B) {
@@ -782,7 +795,8 @@ __device__ void gate_finish(const TcArgs& a, const Phase& ph, const Task& T, uin
 // and the target bytes.  Loading a target in the loop cost an L2 round trip
 // per group (the acquire of the phase counters empties L1): 13,000 to 20,000
 // cycles per head task against about 4,000 for a gate task's epilogue.
-constexpr int kHeadMaxGroups = 8;  // 4-sequence groups of one warp (INF: two targets each)
+// 4-sequence groups of one warp (unperturbed: two targets each)
+__host__ __device__ constexpr int head_targets(bool inf) { return inf ? 16 : 8; }
 
 struct HeadPre {
   float bo[4], dbo[4];
@@ -799,7 +813,7 @@ __device__ __forceinline__ void head_prepare(const TcArgs& a, const Phase& ph, c
   const Layout& L = s.lay;
   const int lane = threadIdx.x & 31;
   const int bq = lane & 3, r4 = lane >> 2;
-  G.sh = epi_share<EPI>(g, ew);
+  G.sh = epi_share<INF, EPI>(g, T.p_valid, ew);
   G.on = G.sh.p < T.p_valid;
   if (!G.on) return;
   const float* th = s.params + (int64_t)T.e * L.P;
@@ -812,10 +826,10 @@ __device__ __forceinline__ void head_prepare(const TcArgs& a, const Phase& ph, c
 #pragma unroll
   for (int k = 0; k < 4; ++k) G.tgt[k] = 0u;
 #pragma unroll
-  for (int j = 0; j < kHeadMaxGroups; ++j) {
+  for (int j = 0; j < head_targets(INF); ++j) {
     const int b = 4 * (G.sh.part + (INF ? j >> 1 : j) * G.sh.parts) + bq;
-    // unperturbed: the sequences of blocks col_c(p) and col_d(p)
-    const int q = INF ? inf_seq(g, T.grp, j & 1 ? col_d(G.sh.p) : col_c(G.sh.p), b) : b;
+    // unperturbed: the sequences of blocks 2p and 2p + 1
+    const int q = INF ? inf_seq(g, T.grp, 2 * G.sh.p + (j & 1), b) : b;
     if (b < g.Bp && q < s.B) {
       const int64_t o = seq_offset(s, T.e, INF ? 0 : i, q) + t + 1;
       if (SOMA_CHECK((size_t)o < a.n_bytes, a.status))
@@ -866,12 +880,12 @@ __device__ bool head_epilogue(const TcArgs& a, const Phase& ph, const Task& T, u
   if (G.on) {
     const int p = G.sh.p, i = T.grp * g.P + p;
     // perturbed: lanes (e, i, +) and (e, i, -) for sequence b; unperturbed:
-    // lane (e, 0, +) for the sequences of blocks col_c(p) and col_d(p)
+    // lane (e, 0, +) for the sequences of blocks 2p and 2p + 1
     const int64_t lane_plus = INF ? (int64_t)T.e * 2 : ((int64_t)T.e * s.n_pert + i) * 2;
-    const uint32_t cC = (uint32_t)(col_c(p) * g.Bp), cD = (uint32_t)(col_d(p) * g.Bp);
+    const uint32_t cC = (uint32_t)(blk_c<INF>(p) * g.Bp), cD = (uint32_t)(blk_d<INF>(p) * g.Bp);
     const int step = 4 * G.sh.parts;
 #pragma unroll
-    for (int j0 = 0; j0 < (INF ? kHeadMaxGroups / 2 : kHeadMaxGroups); j0 += 2) {
+    for (int j0 = 0; j0 < 8; j0 += 2) {
       const int b0 = 4 * G.sh.part + j0 * step;
       if (b0 >= g.Bp) break;
       // [group][k]: logits of row r4 + 8 k, sequence b0 + h step + bq; a second
@@ -940,7 +954,7 @@ __device__ bool head_epilogue(const TcArgs& a, const Phase& ph, const Task& T, u
 #pragma unroll
           for (int sg = 0; sg < 2; ++sg) {
             const int j = 2 * (j0 + h) + sg;
-            const int q = inf_seq(g, T.grp, sg ? col_d(p) : col_c(p), b);
+            const int q = inf_seq(g, T.grp, 2 * p + sg, b);
             const int y = (int)((G.tgt[j >> 2] >> (8 * (j & 3))) & 255u) - vq - r4;
             if (q < s.B && y >= 0 && y < 32 && (y & 7) == 0 &&
                 SOMA_CHECK((size_t)((lane_plus * s.B_mem + s.b0 + q) * (int64_t)s.T + t) < a.n_ply,
@@ -978,7 +992,7 @@ __device__ bool head_epilogue(const TcArgs& a, const Phase& ph, const Task& T, u
     const int pb = idx >> 1;
     const int pp = pb / g.Bp, b = pb % g.Bp;
     // the partials' lane and sequence (see the target logits above)
-    const int qs = INF ? inf_seq(g, T.grp, sgn ? col_d(pp) : col_c(pp), b) : b;
+    const int qs = INF ? inf_seq(g, T.grp, 2 * pp + sgn, b) : b;
     if (qs >= s.B) continue;
     const float2* q = red + (size_t)idx * 4;
     const float M = fmaxf(fmaxf(q[0].x, q[1].x), fmaxf(q[2].x, q[3].x));
@@ -1004,10 +1018,10 @@ __device__ __forceinline__ uint8_t* align1024(uint8_t* p) {
 // cooperative), Warps<INF, EPI>::threads threads.  The CTAs share the tasks of phases
 // 0 .. T through the task counter.
 // SPARSE: sparse probes; INF: the unperturbed layout (eps = 0, one sign).
-template <bool SPARSE, bool INF, int EPI>
+template <bool SPARSE, bool INF, int EPI, int STAGES>
 __global__ void __launch_bounds__((Warps<INF, EPI>::threads), 1)
 tc_persistent_kernel(const TcArgs a) {
-  constexpr int kEpi = EPI, kFirstEpi = Warps<INF, EPI>::epi0, kStages = ring_stages(INF);
+  constexpr int kEpi = EPI, kFirstEpi = Warps<INF, EPI>::epi0, kStages = STAGES;
   extern __shared__ uint8_t dyn_smem[];
   const TcGeom& g = a.g;
   const Sweep& s = a.sw;
@@ -1104,6 +1118,9 @@ tc_persistent_kernel(const TcArgs a) {
         break;
       }
       const Phase ph = make_phase(a, t);
+      // unperturbed: the row blocks the group has
+      const uint32_t b_bytes =
+          INF ? (uint32_t)(inf_blocks(g, T.grp) * g.Bp / 8) * kSbo : SL.b_bytes;
       // the operand rows other CTAs wrote (generic proxy) before the
       // fetcher's acquire are read here by bulk copies (async proxy)
       asm volatile("fence.proxy.async.global;" ::: "memory");
@@ -1117,14 +1134,14 @@ tc_persistent_kernel(const TcArgs a) {
             break;
           }
           uint8_t* slot = smem + q * SL.bytes;
-          if (lane == 0) mbar_arrive_expect_tx(&ctl->full[q], kTileA + SL.b_bytes);
+          if (lane == 0) mbar_arrive_expect_tx(&ctl->full[q], kTileA + b_bytes);
           __syncwarp();
           if (lane < 2) {
             uint8_t* dst = lane == 0 ? slot + SL.a_off : slot + SL.b_off;
             const bool xs = !T.head && st < g.Sx;  // an embedding-part stage
             const uint8_t* src = lane == 0 ? T.a + (size_t)st * kTileA
-                                           : (xs ? T.bx : T.b) + (size_t)st * g.G * g.tileB + SL.b_src;
-            const uint32_t nb = lane == 0 ? kTileA : SL.b_bytes;
+                                           : (xs ? T.bx : T.b) + (size_t)st * g.G * g.tileB;
+            const uint32_t nb = lane == 0 ? kTileA : b_bytes;
             const uint8_t* gbase =
                 lane == 1 ? (xs ? a.xall : ph.op_in) : (T.head ? a.wo16 : a.w16);
             const size_t gsize =
@@ -1160,7 +1177,7 @@ tc_persistent_kernel(const TcArgs a) {
       // W covers the P probes of the group (2 Bp P columns); a group with
       // one valid probe still multiplies the whole window (the rows of the
       // missing probe are zero)
-      const uint32_t idesc_w = idesc_f16_f32(128, 2 * g.Bp * g.P);
+      const uint32_t idesc_g = idesc_f16_f32(128, INF ? 128 : 2 * g.Bp * g.P);
       // descriptors of slot 0; slot q is q * SL.bytes further
       const uint64_t d0 = smem_desc(smem_u32(smem), kLbo, kSbo);
       const uint32_t hi = (uint32_t)(d0 >> 32);
@@ -1168,8 +1185,8 @@ tc_persistent_kernel(const TcArgs a) {
       const uint32_t slot_step = SL.bytes >> 4;
       const uint32_t a_lo0 = lo0 + (SL.a_off >> 4), b_lo0 = lo0 + (SL.b_off >> 4);
       const uint32_t grp_step = kSbo >> 4;                     // 8 operand rows
-      // the W window starts at row Bp of the group tile
-      const uint32_t w_row = (uint32_t)(g.Bp / 8) * grp_step - (SL.b_src >> 4);
+      // the W window starts at row Bp of the group tile (unperturbed: row 0)
+      const uint32_t w_row = INF ? 0u : (uint32_t)(g.Bp / 8) * grp_step;
       const uint32_t z1_row = (uint32_t)(4 * g.Bp / 8) * grp_step;
       const uint32_t dz1 = (uint32_t)(2 * g.Bp);
       RingPos<kStages> rp = {0u, 0u, 0u};
@@ -1184,7 +1201,10 @@ tc_persistent_kernel(const TcArgs a) {
                                                    (uint32_t)((k >> 1) - 1) & 1u, abort, status)))
           break;
         tc_fence_after();
-        const uint32_t d = tmem + (uint32_t)buf * kAccCols;
+        const uint32_t d = tmem + (uint32_t)buf * acc_cols(INF);
+        // unperturbed: as many columns as the group has sequences, in blocks
+        const uint32_t idesc_w =
+            INF ? idesc_f16_f32(128, inf_blocks(g, T.grp) * g.Bp) : idesc_g;
         const int np = do_z ? T.p_valid : 0;
         bool ok;
         if (np == 2)
@@ -1354,7 +1374,7 @@ tc_persistent_kernel(const TcArgs a) {
       {
         const int buf = k & 1;
         const size_t c = (size_t)T.e * g.G + T.grp;
-        const uint32_t tacc = tmem + (uint32_t)buf * kAccCols;
+        const uint32_t tacc = tmem + (uint32_t)buf * acc_cols(INF);
         if (!SOMA_CHECK(c < (size_t)g.n_experts * g.G, status)) {
           alive = false;
           break;
@@ -1369,7 +1389,7 @@ tc_persistent_kernel(const TcArgs a) {
           alive = head_epilogue<INF, EPI>(a, ph, T, tacc, q4, ew, G, red, &ctl->red_bar, &red_use, abort);
           if (!__all_sync(0xffffffffu, alive)) break;
         } else {
-          GatePre<EPI> G;
+          GatePre<INF, EPI> G;
           gate_prepare<INF, EPI>(a, ph, T, q4, ew, G);
           alive = wait_or_abort(&ctl->acc_full[buf], (uint32_t)(k >> 1) & 1u, abort, status);
           if (!__all_sync(0xffffffffu, alive)) break;
@@ -1417,8 +1437,8 @@ __device__ void xpart_block(const TcArgs& a, uint8_t* xall, int t, int blk, int 
     __align__(16) __half v[8];
     const int k0 = kKt * st + 8 * kc;
     if constexpr (INF) {
-      // row blocks 1..4: the embeddings of four blocks of sequences; 0, 5: zero
-      const int q = blkr >= 1 && blkr <= 4 ? inf_seq(g, grp, blkr - 1, b) : s.B;
+      // row block j: the embeddings of the group's block j of sequences
+      const int q = inf_seq(g, grp, blkr, b);
       float x[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
       if (q < s.B && SOMA_CHECK((size_t)seq_offset(s, e, 0, q) + t < a.n_bytes, a.status)) {
         const int y = s.bytes[seq_offset(s, e, 0, q) + t];
@@ -1778,7 +1798,7 @@ size_t kernel_smem_bytes(const TcGeom& g) {
   // ring slots, the control block (1 KB), the head's reduction buffer
   // [P][Bp][2][4] float2 and alignment slack
   const size_t red = (size_t)g.P * g.Bp * 2 * 4 * sizeof(float2);
-  return (size_t)ring_stages(g.inf != 0) * stage_layout(g).bytes + 1024 + red + 1024;
+  return (size_t)ring_stages(g) * stage_layout(g).bytes + 1024 + red + 1024;
 }
 
 }  // namespace
@@ -1820,14 +1840,27 @@ TcGeom make_tc_geom(const Layout& lay, int n_experts, int n_pert, int B, int T, 
   g.Bm = B_mem;
   g.T = T;
   g.inf = 0;
+  g.blocks = 0;
   return g;
 }
 
+// SMs of a GB300; a plan's sizes do not depend on the current device.
+constexpr int kPlanSms = 152;
+
 TcGeom make_tc_geom_inf(const Layout& lay, int n_experts, int B, int T) {
   TcGeom g = make_tc_geom(lay, n_experts, 1, 32, T, B);
-  g.P = 2;
-  g.G = (B + kInfGroupSeqs - 1) / kInfGroupSeqs;
-  g.rowsB = 3 * g.Bp * g.P;
+  // Groups of 8 blocks copy and multiply the most per W tile, groups of 4 make
+  // twice the tasks.  8 once they alone give every SM a task.  Measured, time
+  // with 4 over time with 8 by the tasks of a phase with 8: 0.81 to 0.94 at 46
+  // to 138, 0.89 (8 experts, H = 480, 256 sequences) at 144, 1.09 to 1.22 at
+  // 184 to 256, 1.01 to 1.22 above; routed inference over 8 experts of H = 480,
+  // 1,024 requests (432 tasks): 7.84 -> 6.80 ms.
+  const int64_t tasks8 = (int64_t)n_experts * (g.MT + 2) * ((B + 8 * g.Bp - 1) / (8 * g.Bp));
+  g.blocks = tasks8 > kPlanSms ? kInfBlocks : kInfBlocks / 2;
+  g.P = g.blocks / 2;
+  const int blocks = (B + g.Bp - 1) / g.Bp;
+  g.G = (blocks + g.blocks - 1) / g.blocks;
+  g.rowsB = g.Bp * (blocks < g.blocks ? blocks : g.blocks);
   g.tileB = (uint32_t)g.rowsB * kKt * 2;
   g.B = B;
   g.inf = 1;
@@ -1862,12 +1895,13 @@ cudaError_t launch_forward_tc(const Sweep& s, const TcGeom& g, const TcBuffers& 
                               cudaStream_t stream) {
   const size_t smem = kernel_smem_bytes(g);
   const int epi = g.inf ? kInfEpi : epi_warps_for(g, s.sparse != 0, g.n_experts * (g.MT + 2) * g.G);
-  auto kernel = g.inf ? tc_persistent_kernel<false, true, kInfEpi>
+  auto kernel = g.inf ? (ring_stages(g) == 6 ? tc_persistent_kernel<false, true, kInfEpi, 6>
+                                             : tc_persistent_kernel<false, true, kInfEpi, 4>)
                 : epi == 16
-                    ? (s.sparse ? tc_persistent_kernel<true, false, 16>
-                                : tc_persistent_kernel<false, false, 16>)
-                    : (s.sparse ? tc_persistent_kernel<true, false, 8>
-                                : tc_persistent_kernel<false, false, 8>);
+                    ? (s.sparse ? tc_persistent_kernel<true, false, 16, 5>
+                                : tc_persistent_kernel<false, false, 16, 5>)
+                    : (s.sparse ? tc_persistent_kernel<true, false, 8, 5>
+                                : tc_persistent_kernel<false, false, 8, 5>);
   const int threads = g.inf ? Warps<true, kInfEpi>::threads
                             : epi == 16 ? Warps<false, 16>::threads : Warps<false, 8>::threads;
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,

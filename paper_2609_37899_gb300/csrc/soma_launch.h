@@ -27,20 +27,21 @@ int sm_count();
 // eps^2 dhat per probe, forward_tc.cu).
 //
 // The unperturbed layout (inf = 1: evaluation and routed inference, eps = 0,
-// one sign) uses the same tile shape, but the four row blocks that the W
-// product reads hold four blocks of Bp = 32 different sequences, so a group
-// is 128 sequences and every MMA column does useful work; G groups cover
-// the whole batch in one sweep.
+// one sign) has no probe tiles: a group is up to 4 or 8 blocks of Bp = 32 sequences,
+// its tile their rows, its accumulator one column per sequence, and a task's
+// MMAs and copies take as many blocks as the group has; G groups cover the
+// whole batch in one sweep.
 struct TcGeom {
   int E, H, Ep, Hp, S, Sx, Sh, MT, Bp, P, G, rowsB;
   uint32_t tileB;  // bytes of one operand group tile of one stage
   int n_experts, n_pert, B, T;
   int Bm;          // sequences of the whole batch (the loss partials); B <= 64 of them per sweep
   int inf;         // the unperturbed layout
+  int blocks;      // its sequence blocks per group (4 or 8)
 };
 
-// Sequences of one group of the unperturbed layout.
-constexpr int kInfGroupSeqs = 128;
+// Most sequence blocks of one group of the unperturbed layout.
+constexpr int kInfBlocks = 8;
 
 struct TcSizes {
   size_t w16, wo16, op, cst, pm, ply, zb, cnt, xall;
