@@ -47,18 +47,9 @@ TRAFFIC = {
     # profiles/tc_persistent_kernel_soma_n2.md: one persistent launch of the
     # SOMA N=2 shapes at T=16 (17 phases) captured; per phase, scaled by the
     # T + 1 phases of a launch
-    "soma_n2": {"bytes_per_phase": (2194.885e6 + 869.94816e6) / 17,
+    "soma_n2": {"bytes_per_phase": (2200.845824e6 + 870.040064e6) / 17,
                 "files": ["forward_tc.cu", "tc_primitives.cuh", "soma_device.cuh"],
-                "source_hash": "97f08f55d5cc3326"},
-    # profiles/res_kernel_soma_n256.md: one full-size launch (T=512)
-    "soma_n256": {"bytes_per_launch": 39.452672e6 + 2048,
-                  "files": ["resident.cu", "tc_primitives.cuh", "soma_device.cuh"],
-                  "source_hash": "7cc9de59fd25da8c"},
-    # profiles/body_tc_kernel_body_n256.md: one full-size launch (T=512)
-    "body_n256": {"bytes_per_launch": 36.546304e6,
-                  "files": ["body_tc.cu", "body_device.cuh", "tc_primitives.cuh",
-                            "soma_device.cuh"],
-                  "source_hash": "aed1fa16ae461890"},
+                "source_hash": "ee8ef0435f95da87"},
 }
 
 
@@ -793,8 +784,9 @@ def body_arm(args):
                            "replica(s), no collective",
         },
         "roofline": {
-            "bound": "tensor", "kernel": "body_tc_kernel (tcgen05, one CTA per probe pair and "
-                                         "16-sequence chunk, the whole recurrence resident; "
+            "bound": "tensor", "kernel": "body_tc_kernel (tcgen05, two streams (probe pair, "
+                                         "16-sequence chunk) per CTA, the whole recurrence "
+                                         "resident; "
                                          "its time includes the decode and the loss)",
             "achieved": achieved, "peak": tensor_peak, "unit": "TFLOP/s",
             "frac": (achieved / tensor_peak) if achieved else None, "traffic": traffic,
