@@ -267,6 +267,13 @@ int soma_debug_probe(uint64_t seed, uint64_t step, int expert, int pert, int pro
  *   returns; the context stays usable.  This is the path every kernel of the
  *   library takes when one of its waits runs out. */
 int soma_debug_wait_timeout(uint32_t max_polls, void* stream);
+/* soma_debug_warp_wait: one warp waits as the LSTM kernels' warps do, its even
+ *   lanes on a barrier whose phase has completed, its odd lanes on one that
+ *   nothing completes (mixed != 0), or all on the completed one.  got (device
+ *   int32 [32]) receives each lane's answer, the same in every lane: 1 without
+ *   and 0 with the mix, which also records SOMA_ERR_TIMEOUT after max_polls
+ *   polls (1 .. 2^22). */
+int soma_debug_warp_wait(int mixed, uint32_t max_polls, int* got, void* stream);
 /* soma_debug_tc_gemm: d[128][n] = a[128][k] * b[n][k]^T (fp16 inputs as
  *   uint16 bit patterns, row-major; fp32 output) through the same shared-
  *   memory descriptors, tcgen05.mma and tensor-memory read-back as the

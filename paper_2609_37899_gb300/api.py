@@ -133,6 +133,7 @@ def _open(path: str):
                                                  ctypes.POINTER(soma_estimate_options), f32, u64,
                                                  u64, vp, i32, i32, vp, vp, vp, sz, vp])
         _sig(L, "soma_debug_wait_timeout", i32, [ctypes.c_uint32, vp])
+        _sig(L, "soma_debug_warp_wait", i32, [i32, ctypes.c_uint32, vp, vp])
         bd = soma_body_dims
         _sig(L, "soma_body_param_count", i64, [bd])
         _sig(L, "soma_body_workspace_bytes", sz, [bd, i32, i32, i32, i32])
@@ -352,6 +353,14 @@ def debug_probe(seed: int, step: int, expert: int, probe: int, kind: str, p0: in
 def debug_wait_timeout(max_polls: int, stream=None):
     """Launch a kernel whose bounded wait runs out (see soma_api.h)."""
     _check(lib().soma_debug_wait_timeout(max_polls, _stream(stream)), "soma_debug_wait_timeout")
+
+
+def debug_warp_wait(mixed: bool, max_polls: int, device="cuda", stream=None) -> torch.Tensor:
+    """Each lane's answer [32] from the kernels' warp-wide wait (see soma_api.h)."""
+    got = torch.full((32,), -1, dtype=torch.int32, device=device)
+    _check(lib().soma_debug_warp_wait(int(mixed), max_polls, _dev(got, torch.int32, "got"),
+                                      _stream(stream)), "soma_debug_warp_wait")
+    return got
 
 
 def debug_tc_gemm(a: torch.Tensor, b: torch.Tensor, stream=None,

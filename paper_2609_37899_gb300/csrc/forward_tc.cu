@@ -294,7 +294,8 @@ __device__ __forceinline__ void issue_stage(uint32_t d, uint32_t a_lo, uint32_t 
 // stages, tensor memory four probe tiles), acc_full (a buffer's task is
 // accumulated), acc_empty (its epilogue has read it), mma_done (all MMAs of
 // the CTA completed), task_full / task_empty (the task ring).  Every wait is
-// bounded (wait_or_abort, mbar_wait, wait_counter).
+// bounded (warp_wait, mbar_wait, wait_counter): after one that ran out the CTA
+// winds down without issuing further copies or MMAs.
 // ---------------------------------------------------------------------------
 // One task: (expert, row tile, probe group).  For the gate the row tile is
 // 32 hidden units (128 gate rows); for the head it is a 128-row vocabulary
@@ -326,23 +327,6 @@ struct Ctl {
 };
 static_assert(sizeof(Ctl) <= 1024, "the control block sits in the 1 KB before the head buffer");
 
-// A wait that times out records SOMA_ERR_TIMEOUT in the status word and sets
-// the CTA's abort flag; a wait that is still pending sees the flag within 64
-// polls and returns false, so the CTA winds down without issuing further
-// copies or MMAs.  A phase that is already complete costs one poll and no
-// read of the flag.
-__device__ __forceinline__ bool wait_or_abort(uint64_t* bar, uint32_t parity, volatile int* abort,
-                                              int* status) {
-  if (mbar_try_wait(bar, parity)) return true;
-  for (uint32_t n = 1; n < (1u << 22); ++n) {
-    if ((n & 63u) == 0 && *abort) return false;
-    if (mbar_try_wait(bar, parity)) return true;
-  }
-  *abort = 1;
-  atomicCAS(status, 0, kStatusTimeout);
-  return false;
-}
-
 // Ring position of the next stage: shared-memory slot q and the parity of
 // its phase, probe-tile slot zq.
 template <int STAGES>
@@ -371,8 +355,7 @@ __device__ __forceinline__ bool mma_task(uint64_t* full, uint64_t* slot_free, ui
   for (int st = 0; st < nst; ++st) {
     // the whole warp waits, so the descriptor words stay warp-uniform and
     // one elected thread issues
-    const bool ready = wait_or_abort(&full[rp.q], rp.ph, abort, status);
-    if (__any_sync(0xffffffffu, !ready)) return false;
+    if (!warp_wait(&full[rp.q], rp.ph, abort, status)) return false;
     tc_fence_after();
     // the accumulator block, the probe tiles of the slot and the operand
     // windows (rows of 128 bytes per 8-row group step) stay inside their
@@ -473,13 +456,13 @@ __device__ __forceinline__ void decode_task(const TcArgs& a, int gid, int& t, in
 __device__ __forceinline__ int next_task(Ctl* ctl, uint32_t& kt, volatile int* abort, int* status,
                                          int& t, Task& T, bool release = true) {
   const int sl = (int)(kt % kTaskSlots);
-  if (!wait_or_abort(&ctl->task_full[sl], (kt / kTaskSlots) & 1u, abort, status)) return -2;
+  if (!warp_wait(&ctl->task_full[sl], (kt / kTaskSlots) & 1u, abort, status)) return -2;
   const int gid = ctl->task_gid[sl];
   if (gid >= 0) {
     t = ctl->task_t[sl];
     T = ctl->task[sl];
   }
-  __syncwarp(__activemask());
+  __syncwarp();
   if (release && (threadIdx.x & 31) == 0) mbar_arrive(&ctl->task_empty[sl]);
   ++kt;
   return gid;
@@ -863,7 +846,7 @@ __device__ __forceinline__ bool epi_rendezvous(uint64_t* bar, uint32_t* use, vol
                                                int* status) {
   __syncwarp();
   if ((threadIdx.x & 31) == 0) mbar_arrive(bar);
-  const bool ok = wait_or_abort(bar, *use & 1u, abort, status);
+  const bool ok = warp_wait(bar, *use & 1u, abort, status);
   ++*use;
   __syncwarp();
   return ok;
@@ -1081,7 +1064,7 @@ tc_persistent_kernel(const TcArgs a) {
     for (;;) {
       const int sl = (int)(kt % kTaskSlots);
       if (kt >= kTaskSlots &&
-          !wait_or_abort(&ctl->task_empty[sl], ((kt / kTaskSlots) - 1) & 1u, abort, status))
+          !warp_wait(&ctl->task_empty[sl], ((kt / kTaskSlots) - 1) & 1u, abort, status))
         break;
       int gid = 0;
       if (lane == 0) gid = atomicAdd(a.next_task, 1);
@@ -1134,7 +1117,7 @@ tc_persistent_kernel(const TcArgs a) {
           const int q = gs % kStages;
           const uint32_t use = gs / kStages;
           if (gs >= kStages &&
-              !wait_or_abort(&ctl->slot_free[q], (use - 1) & 1u, abort, status)) {
+              !warp_wait(&ctl->slot_free[q], (use - 1) & 1u, abort, status)) {
             done = false;
             break;
           }
@@ -1201,9 +1184,7 @@ tc_persistent_kernel(const TcArgs a) {
         Task T;
         if (next_task(ctl, kt, abort, status, t, T) < 0) break;
         const int buf = k & 1;
-        if (k >= 2 &&
-            __any_sync(0xffffffffu, !wait_or_abort(&ctl->acc_empty[buf],
-                                                   (uint32_t)((k >> 1) - 1) & 1u, abort, status)))
+        if (k >= 2 && !warp_wait(&ctl->acc_empty[buf], (uint32_t)((k >> 1) - 1) & 1u, abort, status))
           break;
         tc_fence_after();
         const uint32_t d = tmem + (uint32_t)buf * acc_cols(INF);
@@ -1250,9 +1231,8 @@ tc_persistent_kernel(const TcArgs a) {
       if (next_task(ctl, kt, abort, status, t, T, false) < 0) break;
       const size_t c = (size_t)T.e * g.G + T.grp;
       const int sl = k % kTaskSlots;
-      const bool fin = wait_or_abort(&ctl->task_done[sl], (uint32_t)(k / kTaskSlots) & 1u, abort,
-                                     status);
-      if (__any_sync(0xffffffffu, !fin) || !SOMA_CHECK(c < (size_t)g.n_experts * g.G, status))
+      if (!warp_wait(&ctl->task_done[sl], (uint32_t)(k / kTaskSlots) & 1u, abort, status) ||
+          !SOMA_CHECK(c < (size_t)g.n_experts * g.G, status))
         break;
       if (lane == 0) {
         __threadfence();
@@ -1327,13 +1307,11 @@ tc_persistent_kernel(const TcArgs a) {
             const int q = gs % kStages;
             const int zq = gs % kZSlots;
             const uint32_t zuse = gs / kZSlots;
-            // after an abort the generators stop: an arrival on a phase that
-            // can no longer complete would overfill it
-            if (gs >= kZSlots &&
-                !wait_or_abort(&ctl->z_free[zq], (zuse - 1) & 1u, abort, status)) {
-              alive = false;
-              break;
-            }
+            // the vote on this wait comes with the warp's barrier before the
+            // arrival; here it would delay the store (sparse SOMA N=2 at T = 64:
+            // 8.28 ms without any vote, 8.33 so, 8.41 here)
+            const bool ok =
+                gs < kZSlots || lane_wait(&ctl->z_free[zq], (zuse - 1) & 1u, abort, status);
             tc_fence_after();
             if (active &&
                 SOMA_CHECK(kZCol0 + 64u * (uint32_t)zq + 32u * pz + 32u <= kTmemCols, status)) {
@@ -1351,6 +1329,12 @@ tc_persistent_kernel(const TcArgs a) {
               tmem_wait_st();
             }
             tc_fence_before();
+            // after an abort the generators stop: an arrival on a phase that
+            // can no longer complete would overfill it
+            if (__any_sync(0xffffffffu, !ok)) {
+              alive = false;
+              break;
+            }
             __syncwarp();
             if (lane == 0) mbar_arrive(&ctl->full[q]);
           }
@@ -1388,16 +1372,16 @@ tc_persistent_kernel(const TcArgs a) {
         if (T.head) {
           HeadPre G;
           head_prepare<INF, EPI>(a, ph, T, q4, ew, G);
-          alive = wait_or_abort(&ctl->acc_full[buf], (uint32_t)(k >> 1) & 1u, abort, status);
-          if (!__all_sync(0xffffffffu, alive)) break;
+          alive = warp_wait(&ctl->acc_full[buf], (uint32_t)(k >> 1) & 1u, abort, status);
+          if (!alive) break;
           tc_fence_after();
           alive = head_epilogue<INF, EPI>(a, ph, T, tacc, q4, ew, G, red, &ctl->red_bar, &red_use, abort);
-          if (!__all_sync(0xffffffffu, alive)) break;
+          if (!alive) break;
         } else {
           GatePre<INF, EPI> G;
           gate_prepare<INF, EPI>(a, ph, T, q4, ew, G);
-          alive = wait_or_abort(&ctl->acc_full[buf], (uint32_t)(k >> 1) & 1u, abort, status);
-          if (!__all_sync(0xffffffffu, alive)) break;
+          alive = warp_wait(&ctl->acc_full[buf], (uint32_t)(k >> 1) & 1u, abort, status);
+          if (!alive) break;
           tc_fence_after();
           gate_finish<INF, EPI>(a, ph, T, tacc, q4, G);
         }

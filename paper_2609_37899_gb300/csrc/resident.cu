@@ -658,10 +658,13 @@ __global__ void __launch_bounds__((EW + 1) * 32, EW == 8 ? 2 : 1) res_kernel(con
         }
       }
     };
+    // This lane's answer: the caller votes on it.  No lane leaves before the vote,
+    // so after a wait that ran out the accumulators are read all the same (in
+    // bounds, whatever they hold).
     auto head_epilogue = [&](int t) -> bool {
       const uint32_t hb = g.lag ? (uint32_t)t & 1u : 0u;
       const uint32_t par = g.lag ? (uint32_t)(t >> 1) & 1u : (uint32_t)t & 1u;
-      if (!res_wait(&ctl->head_bar[hb], par, abort, a.status)) return false;
+      const bool ok = res_wait(&ctl->head_bar[hb], par, abort, a.status);
       tc_fence_after();
       const uint32_t tq = tq0 + g.hcol + hb * 8u * g.Bp;
       float2* rd = red + (t & 1) * 16 * g.Bp;
@@ -679,7 +682,7 @@ __global__ void __launch_bounds__((EW + 1) * 32, EW == 8 ? 2 : 1) res_kernel(con
       if (!g.sep && 4 * sp >= g.Bp && lane == 0) mbar_arrive(&ctl->acc_free);
       __syncwarp();
       if (lane == 0) mbar_arrive(&ctl->red_full[t & 1]);
-      return true;
+      return ok;
     };
     // gates and cells of NG groups; h into the operand of t + 1
     auto gate_groups = [&](auto ng, int c, uint8_t* opn) {

@@ -516,6 +516,13 @@ int soma_debug_wait_timeout(uint32_t max_polls, void* stream) {
   return cuda_status(launch_debug_wait_timeout(max_polls, status, (cudaStream_t)stream));
 }
 
+int soma_debug_warp_wait(int mixed, uint32_t max_polls, int* got, void* stream) {
+  if (!got || max_polls < 1 || max_polls > (1u << 22)) return SOMA_ERR_INVALID_ARG;
+  int* status = status_ptr();
+  if (!status) return SOMA_ERR_CUDA;
+  return cuda_status(launch_debug_warp_wait(mixed, max_polls, got, status, (cudaStream_t)stream));
+}
+
 int soma_debug_rademacher(uint64_t seed, uint64_t step, int expert, int pert, int64_t p0,
                           int64_t count, int8_t* z_out, void* stream) {
   if (!z_out || count < 0 || p0 < 0 || expert < 0 || pert < 0) return SOMA_ERR_INVALID_ARG;

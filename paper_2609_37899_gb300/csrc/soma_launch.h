@@ -85,6 +85,8 @@ cudaError_t launch_sgd_update(float* params, int64_t P, int64_t dense_from, int 
 cudaError_t launch_init(float* params, const Layout& lay, int n_experts, uint64_t seed, float std,
                         cudaStream_t stream);
 cudaError_t launch_debug_wait_timeout(uint32_t max_polls, int* status, cudaStream_t stream);
+cudaError_t launch_debug_warp_wait(int mixed, uint32_t max_polls, int* got, int* status,
+                                   cudaStream_t stream);
 cudaError_t launch_debug_check_fail(int* status, cudaStream_t stream);
 cudaError_t launch_debug_philox(uint64_t seed, const uint32_t* ctr4, uint32_t* out4, int count,
                                 cudaStream_t stream);

@@ -314,6 +314,24 @@ __global__ void debug_wait_timeout_kernel(uint32_t max_polls, int* status) {
     atomicCAS(status, 0, kStatusTimeout);
 }
 
+// One warp waits with the kernels' wait, lane l on a barrier whose phase has
+// completed (mixed == 0, or l even) or on one that nothing completes; got[l] is
+// its answer.
+__global__ void debug_warp_wait_kernel(int mixed, uint32_t max_polls, int* got, int* status) {
+  __shared__ uint64_t bar[2];
+  __shared__ volatile int abort;
+  if (threadIdx.x == 0) {
+    tc::mbar_init(&bar[0], 1);
+    tc::mbar_init(&bar[1], 1);
+    abort = 0;
+    tc::mbar_fence_init();
+    tc::mbar_arrive(&bar[0]);
+  }
+  __syncthreads();
+  got[threadIdx.x] =
+      tc::warp_wait(&bar[mixed ? threadIdx.x & 1 : 0], 0u, &abort, status, max_polls) ? 1 : 0;
+}
+
 // An index check whose condition is false and that guards no access: the
 // reporting path of the checked build (nothing happens in the default one).
 __global__ void debug_check_fail_kernel(int* status) {
@@ -401,6 +419,12 @@ cudaError_t launch_adam_update(float* params, float* m, float* v, const Layout& 
 
 cudaError_t launch_debug_check_fail(int* status, cudaStream_t stream) {
   debug_check_fail_kernel<<<1, 32, 0, stream>>>(status);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_debug_warp_wait(int mixed, uint32_t max_polls, int* got, int* status,
+                                   cudaStream_t stream) {
+  debug_warp_wait_kernel<<<1, 32, 0, stream>>>(mixed, max_polls, got, status);
   return cudaGetLastError();
 }
 

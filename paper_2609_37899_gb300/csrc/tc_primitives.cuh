@@ -14,6 +14,8 @@
 #include <cstdint>
 #include <cuda_fp16.h>
 
+#include "soma_device.cuh"
+
 namespace soma {
 namespace tc {
 
@@ -90,6 +92,43 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity,
   for (uint32_t n = 0; n < max_polls; ++n)
     if (mbar_try_wait(bar, parity)) return true;
   return false;
+}
+
+// The kernels' waits.  One that runs out (`max_polls` polls) records the timeout
+// and sets the CTA's abort flag; one that is still pending sees the flag within
+// 64 polls and gives up too, so every warp leaves its loop.  A phase that is
+// already complete costs one poll and no read of the flag.
+// The polls after the first are a function of their own: in line they lengthen
+// the loops of every role (SOMA N=8 step at T = 128: 20.4 ms, 21.8 with them).
+__device__ __noinline__ inline bool lane_wait_more(uint64_t* bar, uint32_t parity,
+                                                   volatile int* abort, int* status,
+                                                   uint32_t max_polls) {
+  bool done = false;
+  for (uint32_t n = 1; !done && n < max_polls; ++n) {
+    if ((n & 63u) == 0 && *abort) return false;
+    done = mbar_try_wait(bar, parity);
+  }
+  if (!done) {
+    *abort = 1;
+    atomicCAS(status, 0, kStatusTimeout);
+  }
+  return done;
+}
+
+// The calling lane's answer.  After an abort the lanes of a warp may get
+// different ones: the caller votes before any lane leaves, for the others'
+// shuffles, votes and tensor-memory instructions would wait for it without a
+// bound.
+__device__ __forceinline__ bool lane_wait(uint64_t* bar, uint32_t parity, volatile int* abort,
+                                          int* status, uint32_t max_polls = 1u << 22) {
+  return mbar_try_wait(bar, parity) || lane_wait_more(bar, parity, abort, status, max_polls);
+}
+
+// The whole warp's answer, the same in every lane: true once the phase has
+// completed for all of them.
+__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volatile int* abort,
+                                          int* status, uint32_t max_polls = 1u << 22) {
+  return __all_sync(0xffffffffu, lane_wait(bar, parity, abort, status, max_polls));
 }
 
 // ------------------------------------------------------------- bulk copy --
