@@ -1894,7 +1894,7 @@ cudaError_t launch_forward_tc(const Sweep& s, const TcGeom& g, const TcBuffers& 
   const int threads = g.inf ? Warps<true, kInfEpi>::threads
                             : epi == 16 ? Warps<false, 16>::threads : Warps<false, 8>::threads;
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
+                                       kSmemOptIn);
   if (e != cudaSuccess) return e;
   const TcSizes z = tc_sizes(g);
   TcArgs a;
@@ -2003,7 +2003,8 @@ cudaError_t launch_debug_tc_gemm(const void* A, const void* B, float* D, int N, 
                                  int a_in_tmem, int* status, cudaStream_t stream) {
   const size_t smem = (size_t)(128 + N) * K * 2 + 1024;
   cudaError_t e = cudaFuncSetAttribute(debug_tc_gemm_kernel,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (128 + 256) * 256 * 2 + 1024);  // K = N = 256
   if (e != cudaSuccess) return e;
   debug_tc_gemm_kernel<<<1, 128, smem, stream>>>(static_cast<const __half*>(A),
                                                  static_cast<const __half*>(B), D, N, K, a_in_tmem,

@@ -818,8 +818,9 @@ bool res_supported(const Layout& lay, int B) {
 
 template <int EW>
 static cudaError_t launch_res(const ResArgs& a, int pairs, cudaStream_t stream) {
-  cudaError_t e = cudaFuncSetAttribute(
-      res_kernel<EW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)a.g.bytes);
+  cudaError_t e =
+      cudaFuncSetAttribute(res_kernel<EW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           EW == 8 ? (int)kResHalfSmem : kSmemOptIn);
   if (e != cudaSuccess) return e;
   trace_begin(SOMA_TRACE_GATE, stream);
   res_kernel<EW><<<pairs, (EW + 1) * 32, a.g.bytes, stream>>>(a);

@@ -24,7 +24,6 @@ __device__ int g_soma_status[2] = {0, 0};
 namespace {
 
 constexpr int kMaxDevices = 64;
-constexpr int kMaxPert = 12 * 1024;  // coefficients of one expert staged in shared memory
 int* g_status_ptr[kMaxDevices] = {nullptr};
 
 int* status_ptr() {

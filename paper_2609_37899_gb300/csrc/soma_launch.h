@@ -18,6 +18,15 @@ void trace_end(int kind, cudaStream_t stream);
 // SMs of the current device.
 int sm_count();
 
+// Most probes of one expert: their coefficients are staged in shared memory.
+constexpr int kMaxPert = 12 * 1024;
+
+// Dynamic shared memory that a CTA can have (sm_103a).  The limit of a kernel
+// (cudaFuncAttributeMaxDynamicSharedMemorySize) is process-wide and every
+// launcher sets it to one constant per kernel, this or less: set to each call's
+// own size it could be lowered by another thread between a call's setting and
+// its launch.
+constexpr int kSmemOptIn = 227 * 1024;
 
 // ---- tensor-core path ------------------------------------------------------
 // Geometry of one sweep on the tensor cores.  K of the gate GEMM is

@@ -15,6 +15,7 @@ namespace {
 
 constexpr int kUpdThreads = 128;
 constexpr int kUpdParams = kUpdThreads * 32;  // parameters of one block
+constexpr int kUpdSmem = kMaxPert * (int)sizeof(float);  // most dynamic shared memory
 
 // acc += c z for one probe over a run: neg, act are its raw words, in which
 // offset 2J of the run is bit J and offset 2J + 1 is bit J + 16 (reading them
@@ -347,7 +348,7 @@ cudaError_t launch_sgd_update(float* params, int64_t P, int64_t dense_from, int 
   const size_t smem = (size_t)n_pert * sizeof(float);  // plus the 16 KB staging array
   auto kernel = sparse ? sgd_update_kernel<true> : sgd_update_kernel<false>;
   cudaError_t e =
-      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kUpdSmem);
   if (e != cudaSuccess) return e;
   trace_begin(SOMA_TRACE_UPDATE, stream);
   kernel<<<grid, kUpdThreads, smem, stream>>>(params, P, dense_from, n_pert, lr, seed, step, coef);
@@ -401,7 +402,7 @@ cudaError_t launch_probe_adam(float* params, float* m, float* v, int64_t P, int6
   const size_t smem = (size_t)n_pert * sizeof(float);
   auto kernel = sparse ? adam_update_kernel<true> : adam_update_kernel<false>;
   cudaError_t e =
-      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kUpdSmem);
   if (e != cudaSuccess) return e;
   trace_begin(SOMA_TRACE_UPDATE, stream);
   kernel<<<grid, kUpdThreads, smem, stream>>>(params, m, v, P, dense_from, n_experts, n_pert, seed,
