@@ -274,6 +274,11 @@ int soma_debug_wait_timeout(uint32_t max_polls, void* stream);
  *   and 0 with the mix, which also records SOMA_ERR_TIMEOUT after max_polls
  *   polls (1 .. 2^22). */
 int soma_debug_warp_wait(int mixed, uint32_t max_polls, int* got, void* stream);
+/* soma_debug_epilogue_warps: the epilogue warps (8 or 16) that a tensor-core sweep
+ *   of these sizes (batch <= 64) runs on a GPU of `sms` SMs; 0 if the sizes are
+ *   invalid.  Host arithmetic only. */
+int soma_debug_epilogue_warps(soma_dims d, int n_experts, int n_pert, int probe_kind, int batch,
+                              int sms);
 /* soma_debug_tc_gemm: d[128][n] = a[128][k] * b[n][k]^T (fp16 inputs as
  *   uint16 bit patterns, row-major; fp32 output) through the same shared-
  *   memory descriptors, tcgen05.mma and tensor-memory read-back as the

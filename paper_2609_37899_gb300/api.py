@@ -133,6 +133,7 @@ def _open(path: str):
                                                  ctypes.POINTER(soma_estimate_options), f32, u64,
                                                  u64, vp, i32, i32, vp, vp, vp, sz, vp])
         _sig(L, "soma_debug_wait_timeout", i32, [ctypes.c_uint32, vp])
+        _sig(L, "soma_debug_epilogue_warps", i32, [soma_dims, i32, i32, i32, i32, i32])
         _sig(L, "soma_debug_warp_wait", i32, [i32, ctypes.c_uint32, vp, vp])
         bd = soma_body_dims
         _sig(L, "soma_body_param_count", i64, [bd])

@@ -80,7 +80,7 @@ constexpr int kZWarp0 = 4;       // Z generators: a multiple of 4 (TMEM lane qua
 constexpr int kZWarps = 8;       // (probe, lane quarter)
 // Epilogue warps EPI (a multiple of 8: probe or sequence share, lane quarter):
 // 16 in the unperturbed layout, which has no probe tiles and takes the
-// generators' warps; 8 or 16 in the perturbed one (see epi_warps_for).
+// generators' warps; 8 or 16 in the perturbed one (see tc_epilogue_warps).
 constexpr int kInfEpi = 16;
 template <bool INF, int EPI>
 struct Warps {
@@ -1771,18 +1771,6 @@ debug_tc_gemm_kernel(const __half* A, const __half* B, float* D, int N, int K, i
   if (tid < 32) tmem_dealloc(tmem, 512);
 }
 
-// Epilogue warps of a perturbed sweep.  With few stages along K a task's MMAs
-// take less time than its epilogue on 8 warps, and 16 are worth the registers
-// (72 a thread instead of 96); with many stages, or more generator work per stage
-// (sparse probes), the extra warps only compete for issue slots, and with fewer
-// tasks than SMs nothing waits for an epilogue.  Measured, time with 8 over time
-// with 16 (8 experts, 64 probes, 32 sequences), dense: 1.28 at S = 3 stages, 1.22
-// at 5, 1.15 at 7, 1.05 at 8, 0.97 at 9, 0.96 at 16; sparse: 1.25, 1.19, 1.01,
-// 0.96, 0.91, 0.91; 16 to 60 tasks on 152 SMs: 0.97 to 1.00.
-int epi_warps_for(const TcGeom& g, bool sparse, int tasks) {
-  return tasks > sm_count() && g.S <= (sparse ? 7 : 8) ? 16 : 8;
-}
-
 size_t kernel_smem_bytes(const TcGeom& g) {
   // ring slots, the control block (1 KB), the head's reduction buffer
   // [P][Bp][2][4] float2 and alignment slack
@@ -1802,6 +1790,30 @@ int sm_count() {
     cached[dev] = n;
   }
   return cached[dev];
+}
+
+// 8 or 16 epilogue warps.  The warps beyond 8 share a task's 8-sequence chunks (P
+// probes of Bp / 8) with the first 8: with one or two chunks they have none, and
+// what is left of 16 warps is their cost, fewer registers (72 a thread instead of
+// 96) and issue slots taken from the generators.  With more chunks they are worth
+// it while a task's MMAs take less time than its epilogue on 8 warps, that is
+// with few stages S along K, fewer for sparse probes, whose generators do more per
+// stage; with no more tasks than SMs nothing waits for an epilogue.  Measured,
+// time with 8 over time with 16:
+//   1, 2 chunks  dense 0.85 to 0.96, sparse 0.82 to 0.93, at S = 3 to 12;
+//   3, 4 chunks  dense 1.12 to 1.19 at S = 3, 1.06 at 5, 0.95 to 1.09 at 6, 0.92 at 8;
+//                sparse 1.10 to 1.19 at 3, 0.96 at 5, 0.87 to 0.92 at 6;
+//   5 to 8       dense 1.07 to 1.32 at 3, 1.04 to 1.25 at 5, 1.01 to 1.19 at 6, 0.94
+//                to 1.14 at 8, 0.92 to 1.04 at 9, 0.93 to 0.96 at 12;
+//                sparse 1.06 to 1.29 at 3, 1.05 to 1.21 at 5, 0.98 to 1.17 at 6,
+//                0.84 to 0.95 at 8, 0.80 to 0.88 at 9 and 12;
+//   16 to 60 tasks on 152 SMs: 0.97 to 1.00.
+int tc_epilogue_warps(const TcGeom& g, bool sparse, int sms) {
+  const int64_t tasks = (int64_t)g.n_experts * (g.MT + 2) * g.G;
+  const int chunks = g.P * (g.Bp / 8);
+  if (tasks <= sms || chunks <= 2) return 8;
+  const int most = chunks <= 4 ? (sparse ? 4 : 5) : (sparse ? 6 : 8);
+  return g.S <= most ? 16 : 8;
 }
 
 TcGeom make_tc_geom(const Layout& lay, int n_experts, int n_pert, int B, int T, int B_mem) {
@@ -1883,7 +1895,7 @@ TcSizes tc_sizes(const TcGeom& g) {
 cudaError_t launch_forward_tc(const Sweep& s, const TcGeom& g, const TcBuffers& tb, int* status,
                               cudaStream_t stream) {
   const size_t smem = kernel_smem_bytes(g);
-  const int epi = g.inf ? kInfEpi : epi_warps_for(g, s.sparse != 0, g.n_experts * (g.MT + 2) * g.G);
+  const int epi = g.inf ? kInfEpi : tc_epilogue_warps(g, s.sparse != 0, sm_count());
   auto kernel = g.inf ? (ring_stages(g) == 6 ? tc_persistent_kernel<false, true, kInfEpi, 6>
                                              : tc_persistent_kernel<false, true, kInfEpi, 4>)
                 : epi == 16

@@ -515,6 +515,14 @@ int soma_debug_wait_timeout(uint32_t max_polls, void* stream) {
   return cuda_status(launch_debug_wait_timeout(max_polls, status, (cudaStream_t)stream));
 }
 
+int soma_debug_epilogue_warps(soma_dims d, int n_experts, int n_pert, int probe_kind, int batch,
+                              int sms) {
+  if (!dims_ok(d) || !sizes_ok(n_experts, n_pert, batch, 1) || batch > kTcMaxBatch || sms < 1)
+    return 0;
+  const TcGeom g = make_tc_geom(make_layout(d.embed, d.hidden), n_experts, n_pert, batch, 1, batch);
+  return tc_epilogue_warps(g, probe_kind == SOMA_PROBE_SPARSE, sms);
+}
+
 int soma_debug_warp_wait(int mixed, uint32_t max_polls, int* got, void* stream) {
   if (!got || max_polls < 1 || max_polls > (1u << 22)) return SOMA_ERR_INVALID_ARG;
   int* status = status_ptr();

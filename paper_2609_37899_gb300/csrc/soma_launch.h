@@ -70,6 +70,8 @@ struct TcBuffers {
 };
 
 TcGeom make_tc_geom(const Layout& lay, int n_experts, int n_pert, int B, int T, int B_mem);
+// Epilogue warps (8 or 16) of the persistent kernel for a perturbed sweep.
+int tc_epilogue_warps(const TcGeom& g, bool sparse, int sms);
 // The unperturbed layout for B sequences per expert (all in one sweep).
 TcGeom make_tc_geom_inf(const Layout& lay, int n_experts, int B, int T);
 // Sequences of one tensor-core sweep; a larger batch runs in chunks of this many.
