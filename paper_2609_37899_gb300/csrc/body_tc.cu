@@ -328,11 +328,16 @@ __global__ void __launch_bounds__(NS * kWarps * 32, 1) body_tc_kernel(const Body
   const int e = (int)(cta / per_e), s0 = (int)(cta % per_e) * NS;
   const int st = warp / kWarps, ew = warp % kWarps;  // the warp's stream, its number in it
   const int stid = tid % kStThr;
-  const bool live = s0 + st < streams;
   const int i = min(s0 + st, streams - 1) / a.chunks, chunk = min(s0 + st, streams - 1) % a.chunks;
   const int64_t pair = (int64_t)e * a.n_pert + i;
   const int b0c = chunk * kBp;
   const int rows = min(kBp, a.B - b0c);
+  // the stream's sequences, its expert's parameters and its NLL partials lie inside
+  // the caller's buffers
+  const bool live = s0 + st < streams &&
+                    SOMA_CHECK(chunk < a.chunks && b0c < a.B &&
+                                   pair < (int64_t)a.n_experts * a.n_pert,
+                               a.status);
   const int D = a.blocks;
   const float eps = a.eps;
   const bool do_z = eps != 0.f;

@@ -351,7 +351,7 @@ __device__ __forceinline__ bool mma_task(uint64_t* full, uint64_t* slot_free, ui
                                          uint32_t a_lo0, uint32_t b_lo0, uint32_t slot_step,
                                          uint32_t hi, uint32_t w_row, uint32_t z1_row,
                                          uint32_t idesc_w, uint32_t idesc_z, uint32_t dz1,
-                                         volatile int* abort, int* status) {
+                                         uint32_t acc_end, volatile int* abort, int* status) {
   for (int st = 0; st < nst; ++st) {
     // the whole warp waits, so the descriptor words stay warp-uniform and
     // one elected thread issues
@@ -360,7 +360,8 @@ __device__ __forceinline__ bool mma_task(uint64_t* full, uint64_t* slot_free, ui
     // the accumulator block, the probe tiles of the slot and the operand
     // windows (rows of 128 bytes per 8-row group step) stay inside their
     // allocations
-    if (!SOMA_CHECK((NP == 0 || (d & 0xFFFFu) + dz1 + (NP >= 2 ? dz1 : 0) <= 2 * kAccCols) &&
+    if (!SOMA_CHECK((d & 0xFFFFu) + idesc_columns(idesc_w) <= acc_end &&
+                        (d & 0xFFFFu) + NP * dz1 <= acc_end &&
                         kZCol0 + 64u * rp.zq + 32u * (NP > 0 ? NP : 1) <= kTmemCols &&
                         rp.q < (uint32_t)STAGES && rp.zq < (uint32_t)kZSlots,
                     status))
@@ -745,16 +746,17 @@ __device__ void gate_finish(const TcArgs& a, const Phase& ph, const Task& T, uin
       const size_t tile_off = (size_t)(out_tile - ph.op_out);
       if (unit_ok &&
           SOMA_CHECK((size_t)(cell - reinterpret_cast<float2*>(a.cst) + b + 1) * 2 <= a.n_cst &&
-                         tile_off + g.tileB <= a.n_op && rE + b < g.rowsB &&
-                         (INF || (rD + b < g.rowsB && rM + b < g.rowsB)) && kk < kKt,
+                         tile_off + g.tileB <= a.n_op && kk < kKt &&
+                         (INF || (rE + b < g.rowsB && rD + b < g.rowsB && rM + b < g.rowsB)),
                      a.status)) {
         cell[b] = make_float2(cp, cm);
         if constexpr (INF) {
           // h of the two blocks into their own rows (the W product's rows)
-          if (inf_seq(g, T.grp, 2 * p, b) < s.B)
+          // (an odd last block has no partner: its rows end the tile)
+          if (inf_seq(g, T.grp, 2 * p, b) < s.B && SOMA_CHECK(rM + b < g.rowsB, a.status))
             *reinterpret_cast<__half*>(out_tile + kmajor_offset(rM + b, kk, kKt)) =
                 __float2half_rn(actp[3] * tp);
-          if (inf_seq(g, T.grp, 2 * p + 1, b) < s.B)
+          if (inf_seq(g, T.grp, 2 * p + 1, b) < s.B && SOMA_CHECK(rD + b < g.rowsB, a.status))
             *reinterpret_cast<__half*>(out_tile + kmajor_offset(rD + b, kk, kKt)) =
                 __float2half_rn(actm[3] * tm);
         } else if (b < s.B) {
@@ -1188,6 +1190,7 @@ tc_persistent_kernel(const TcArgs a) {
           break;
         tc_fence_after();
         const uint32_t d = tmem + (uint32_t)buf * acc_cols(INF);
+        const uint32_t acc_end = (uint32_t)(buf + 1) * acc_cols(INF);  // of the task's buffer
         // unperturbed: as many columns as the group has sequences, in blocks
         const uint32_t idesc_w =
             INF ? idesc_f16_f32(128, inf_blocks(g, T.grp) * g.Bp) : idesc_g;
@@ -1195,13 +1198,13 @@ tc_persistent_kernel(const TcArgs a) {
         bool ok;
         if (np == 2)
           ok = mma_task<2, kStages>(ctl->full, ctl->slot_free, ctl->z_free, rp, T.nst, d, tmem, a_lo0, b_lo0,
-                           slot_step, hi, w_row, z1_row, idesc_w, idesc_z, dz1, abort, status);
+                           slot_step, hi, w_row, z1_row, idesc_w, idesc_z, dz1, acc_end, abort, status);
         else if (np == 1)
           ok = mma_task<1, kStages>(ctl->full, ctl->slot_free, ctl->z_free, rp, T.nst, d, tmem, a_lo0, b_lo0,
-                           slot_step, hi, w_row, z1_row, idesc_w, idesc_z, dz1, abort, status);
+                           slot_step, hi, w_row, z1_row, idesc_w, idesc_z, dz1, acc_end, abort, status);
         else
           ok = mma_task<0, kStages>(ctl->full, ctl->slot_free, ctl->z_free, rp, T.nst, d, tmem, a_lo0, b_lo0,
-                           slot_step, hi, w_row, z1_row, idesc_w, idesc_z, dz1, abort, status);
+                           slot_step, hi, w_row, z1_row, idesc_w, idesc_z, dz1, acc_end, abort, status);
         if (!ok) break;
         if (elect_one()) mma_commit(&ctl->acc_full[buf]);
         __syncwarp();

@@ -193,6 +193,11 @@ __host__ __device__ __forceinline__ uint32_t idesc_f16_f32(int M, int N) {
   return d;
 }
 
+// N of an instruction descriptor: the accumulator columns it writes.
+__host__ __device__ __forceinline__ uint32_t idesc_columns(uint32_t idesc) {
+  return ((idesc >> 17) & 0x3Fu) << 3;
+}
+
 // Descriptor split into its two 32-bit words: the low word holds the start
 // address (bits 0..13, in 16-byte units) and LBO; moving a descriptor by a
 // byte offset d that keeps the address below 256 KB is lo + (d >> 4).
