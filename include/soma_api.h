@@ -274,6 +274,10 @@ int soma_debug_wait_timeout(uint32_t max_polls, void* stream);
  *   and 0 with the mix, which also records SOMA_ERR_TIMEOUT after max_polls
  *   polls (1 .. 2^22). */
 int soma_debug_warp_wait(int mixed, uint32_t max_polls, int* got, void* stream);
+/* soma_debug_activations: differ (device uint64 [3]) receives how many of the
+ *   2^32 floats give other bits with the kernels' sigmoid, tanh and (arguments up
+ *   to 0) softmax term added to 1 than with CUDA's __expf and __fdividef. */
+int soma_debug_activations(uint64_t* differ, void* stream);
 /* soma_debug_epilogue_warps: the epilogue warps (8 or 16) that a tensor-core sweep
  *   of these sizes (batch <= 64) runs on a GPU of `sms` SMs; 0 if the sizes are
  *   invalid.  Host arithmetic only. */

@@ -133,6 +133,7 @@ def _open(path: str):
                                                  ctypes.POINTER(soma_estimate_options), f32, u64,
                                                  u64, vp, i32, i32, vp, vp, vp, sz, vp])
         _sig(L, "soma_debug_wait_timeout", i32, [ctypes.c_uint32, vp])
+        _sig(L, "soma_debug_activations", i32, [vp, vp])
         _sig(L, "soma_debug_epilogue_warps", i32, [soma_dims, i32, i32, i32, i32, i32])
         _sig(L, "soma_debug_warp_wait", i32, [i32, ctypes.c_uint32, vp, vp])
         bd = soma_body_dims
@@ -362,6 +363,15 @@ def debug_warp_wait(mixed: bool, max_polls: int, device="cuda", stream=None) -> 
     _check(lib().soma_debug_warp_wait(int(mixed), max_polls, _dev(got, torch.int32, "got"),
                                       _stream(stream)), "soma_debug_warp_wait")
     return got
+
+
+def debug_activations(device="cuda", stream=None) -> torch.Tensor:
+    """Floats (of all 2^32) whose sigmoid, tanh and softmax term have other bits
+    than with CUDA's own functions [3] (see soma_api.h)."""
+    differ = torch.full((3,), -1, dtype=torch.int64, device=device)
+    _check(lib().soma_debug_activations(_dev(differ, torch.int64, "differ"), _stream(stream)),
+           "soma_debug_activations")
+    return differ
 
 
 def debug_tc_gemm(a: torch.Tensor, b: torch.Tensor, stream=None,

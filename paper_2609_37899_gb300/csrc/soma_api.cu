@@ -515,6 +515,12 @@ int soma_debug_wait_timeout(uint32_t max_polls, void* stream) {
   return cuda_status(launch_debug_wait_timeout(max_polls, status, (cudaStream_t)stream));
 }
 
+int soma_debug_activations(uint64_t* differ, void* stream) {
+  if (!differ) return SOMA_ERR_INVALID_ARG;
+  return cuda_status(launch_debug_activations(reinterpret_cast<unsigned long long*>(differ),
+                                              (cudaStream_t)stream));
+}
+
 int soma_debug_epilogue_warps(soma_dims d, int n_experts, int n_pert, int probe_kind, int batch,
                               int sms) {
   if (!dims_ok(d) || !sizes_ok(n_experts, n_pert, batch, 1) || batch > kTcMaxBatch || sms < 1)

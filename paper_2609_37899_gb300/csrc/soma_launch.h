@@ -96,6 +96,7 @@ cudaError_t launch_sgd_update(float* params, int64_t P, int64_t dense_from, int 
 cudaError_t launch_init(float* params, const Layout& lay, int n_experts, uint64_t seed, float std,
                         cudaStream_t stream);
 cudaError_t launch_debug_wait_timeout(uint32_t max_polls, int* status, cudaStream_t stream);
+cudaError_t launch_debug_activations(unsigned long long* differ, cudaStream_t stream);
 cudaError_t launch_debug_warp_wait(int mixed, uint32_t max_polls, int* got, int* status,
                                    cudaStream_t stream);
 cudaError_t launch_debug_check_fail(int* status, cudaStream_t stream);

@@ -22,9 +22,8 @@ constexpr int kUpdSmem = kMaxPert * (int)sizeof(float);  // most dynamic shared 
 // in raw order saves the spread into natural order).  Each element's additions
 // are single fp32 additions in probe order: the sums keep their bits whatever
 // the grid.
-// Bound: issue.  Dense: the sign selects +-c, one select and one addition
-// (the tests of a word's bits become predicates a byte at a time); sparse: two
-// predicated additions.  Measured on GB300, dense update of 8.3M parameters
+// Bound: issue.  Dense: the sign selects +-c, which is added; sparse: +c or -c is
+// added where the sign and activity bits say so.  Measured on GB300, dense update of 8.3M parameters
 // over 1,024 probes / sparse Adam update of 8.4M over 4 x 64: 1268 / 574 us
 // before, 1000 / 473 us now; signs by integer multiply-add into
 // packed pair additions 1154 / 573 us.
@@ -333,6 +332,25 @@ __global__ void debug_warp_wait_kernel(int mixed, uint32_t max_polls, int* got, 
       tc::warp_wait(&bar[mixed ? threadIdx.x & 1 : 0], 0u, &abort, status, max_polls) ? 1 : 0;
 }
 
+// The activations of tc_primitives.cuh against the same forms with CUDA's __expf
+// and __fdividef: how many of the 2^32 floats differ, for the sigmoid, the tanh
+// and (arguments up to 0) a softmax term added to 1.  Two NaNs count as equal.
+__global__ void debug_activations_kernel(unsigned long long* differ) {
+  unsigned long long n[3] = {0, 0, 0};
+  auto other = [](float a, float b) {
+    return __float_as_uint(a) != __float_as_uint(b) && !(isnan(a) && isnan(b));
+  };
+  const uint64_t step = (uint64_t)gridDim.x * blockDim.x;
+  for (uint64_t u = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; u < (1ull << 32); u += step) {
+    const float x = __uint_as_float((uint32_t)u);
+    n[0] += other(tc::sigmoid_f(x), __fdividef(1.f, 1.f + __expf(-x)));
+    n[1] += other(tc::tanh_f(x), fmaf(__fdividef(1.f, 1.f + __expf(-2.f * x)), 2.f, -1.f));
+    if (!(x > 0.f)) n[2] += other(1.f + tc::exp_term(x), 1.f + __expf(x));
+  }
+  for (int k = 0; k < 3; ++k)
+    if (n[k]) atomicAdd(differ + k, n[k]);
+}
+
 // An index check whose condition is false and that guards no access: the
 // reporting path of the checked build (nothing happens in the default one).
 __global__ void debug_check_fail_kernel(int* status) {
@@ -420,6 +438,13 @@ cudaError_t launch_adam_update(float* params, float* m, float* v, const Layout& 
 
 cudaError_t launch_debug_check_fail(int* status, cudaStream_t stream) {
   debug_check_fail_kernel<<<1, 32, 0, stream>>>(status);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_debug_activations(unsigned long long* differ, cudaStream_t stream) {
+  cudaError_t e = cudaMemsetAsync(differ, 0, 3 * sizeof(*differ), stream);
+  if (e != cudaSuccess) return e;
+  debug_activations_kernel<<<8 * sm_count(), 256, 0, stream>>>(differ);
   return cudaGetLastError();
 }
 
