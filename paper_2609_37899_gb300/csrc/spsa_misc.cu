@@ -20,8 +20,9 @@ constexpr int kUpdSmem = kMaxPert * (int)sizeof(float);  // most dynamic shared 
 // acc += c z for one probe over a run: neg, act are its raw words, in which
 // offset 2J of the run is bit J and offset 2J + 1 is bit J + 16 (reading them
 // in raw order saves the spread into natural order).  Each element's additions
-// are single fp32 additions in probe order: the sums keep their bits whatever
-// the grid.
+// are single fp32 additions in one order, whatever the grid: the groups of four
+// probes i0, i0 + 1, .. in turn and, inside a group, parameter p begins with probe
+// i0 + (p / 32) % 4 and goes round (accumulate_x4).
 // Bound: issue.  Dense: the sign selects +-c, which is added; sparse: +c or -c is
 // added where the sign and activity bits say so.  Measured on GB300, dense update of 8.3M parameters
 // over 1,024 probes / sparse Adam update of 8.4M over 4 x 64: 1268 / 574 us
