@@ -35,7 +35,8 @@
 // probes, 16 x 512 bytes: 161.9 ms with one CTA of 16 epilogue warps per SM and
 // a CTA barrier per timestep, 107.0 ms now (two per SM with a group of four
 // sequences at a time 132 ms; groups in pairs 115; a commit per gate tile 110;
-// the MMA loops without a branch on the tile's place 107).  One expert of E = 32,
+// the MMA loops without a branch on the tile's place 107; the form's own parts
+// known at compile time, 15.8 -> 15.1 ms at T = 64).  One expert of E = 32,
 // H = 64, 8 probes, 4 x 64 bytes: 204 -> 159 us (the merge off the epilogue
 // warps, no barrier).  One MMA of this size occupies the tensor pipe about 46
 // cycles, so the 24 of a gate bound the latter's chain.
@@ -70,7 +71,6 @@ struct ResGeom {
   uint32_t zcol, hcol;  // TMEM columns: probe tiles, head accumulators (gate accumulators at 0)
   uint32_t tmem_cols;   // allocated
   int z_tmem;           // probe tiles in tensor memory (else in shared memory at zg, zo)
-  int lag;              // 1: two head accumulators, the head epilogue runs a timestep behind
   int sep;              // the gate and the head have accumulators of their own
 };
 
@@ -95,8 +95,8 @@ void res_dims(ResGeom& r, const Layout& lay, int B, int T) {
 }
 
 // Shared-memory carve-up; the probe tiles take part unless z_tmem.  The operand
-// has two buffers: MMAs still read one (the head's with lag, those of another
-// gate tile without) while the cells write the other.
+// has two buffers: MMAs still read one (the head's in the one-CTA form, those of
+// another gate tile in the two-CTA form) while the cells write the other.
 void res_carve(ResGeom& r) {
   uint32_t o = 0;
   const uint32_t gate_tile = 128u * r.K * 2, head_tile = 128u * r.Hk * 2;
@@ -125,7 +125,6 @@ uint32_t res_tile_cols(const ResGeom& r) { return 4u * r.Bp; }
 bool make_res_geom_half(ResGeom& r, const Layout& lay, int B, int T) {
   res_dims(r, lay, B, T);
   r.z_tmem = 1;
-  r.lag = 0;
   const uint32_t gate = r.MTg * res_tile_cols(r), head = 2 * res_tile_cols(r);
   const uint32_t z = r.MTg * r.K / 2 + r.Hk;
   r.sep = gate + head + z <= 256;
@@ -140,7 +139,6 @@ bool make_res_geom_half(ResGeom& r, const Layout& lay, int B, int T) {
 ResGeom make_res_geom(const Layout& lay, int B, int T) {
   ResGeom r;
   res_dims(r, lay, B, T);
-  r.lag = 1;
   r.sep = 1;
   r.hcol = r.MTg * res_tile_cols(r);
   r.zcol = r.hcol + 4 * res_tile_cols(r);
@@ -196,6 +194,8 @@ __device__ __forceinline__ uint32_t z_pair_word(const ProbeBits& b, int j, int v
 template <int EW>
 __global__ void __launch_bounds__((EW + 1) * 32, EW == 8 ? 2 : 1) res_kernel(const ResArgs a) {
   constexpr int kThr = (EW + 1) * 32;
+  // timesteps that the head epilogue runs behind (on two accumulators)
+  constexpr int kLag = EW == 16 ? 1 : 0;
   constexpr int kSeqSplit = EW / 8;                        // warps that share a row quarter
   constexpr int kGroups = kResMaxBp / 4 / kSeqSplit;       // 4-sequence groups of one warp
   constexpr int kXChunks = 512 / (EW * 32);                // embedding chunks of one thread
@@ -203,6 +203,8 @@ __global__ void __launch_bounds__((EW + 1) * 32, EW == 8 ? 2 : 1) res_kernel(con
   uint8_t* smem = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(dyn_smem) + 1023) & ~uintptr_t(1023));
   const ResGeom& g = a.g;
+  // what the form decides is known here
+  const bool z_tmem = EW == 8 || g.z_tmem, sep = EW == 16 || g.sep;
   const Sweep& s = a.sw;
   const Layout& L = s.lay;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -256,7 +258,7 @@ __global__ void __launch_bounds__((EW + 1) * 32, EW == 8 ? 2 : 1) res_kernel(con
       }
     }
     ProbeBits zb = {0u, 0u};
-    if (!g.z_tmem && kmax > 0 && do_z) zb = probe_bits(pk, p0, s.sparse);
+    if (!z_tmem && kmax > 0 && do_z) zb = probe_bits(pk, p0, s.sparse);
     if (kmax > 0 && !SOMA_CHECK((size_t)(e * L.P + p0 + kmax) <= a.n_params, a.status)) kmax = 0;
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
@@ -265,9 +267,9 @@ __global__ void __launch_bounds__((EW + 1) * 32, EW == 8 ? 2 : 1) res_kernel(con
       z[j] = ok ? z_half(zb, j) : __float2half_rn(0.f);
     }
     const uint32_t off = m * (128u * g.K * 2) + kmajor_offset(r, k0, g.K);
-    if (SOMA_CHECK(off + 16 <= g.MTg * 128u * g.K * 2 && (g.z_tmem || g.zg + off + 16 <= g.bytes), a.status)) {
+    if (SOMA_CHECK(off + 16 <= g.MTg * 128u * g.K * 2 && (z_tmem || g.zg + off + 16 <= g.bytes), a.status)) {
       *reinterpret_cast<uint4*>(smem + g.wg + off) = *reinterpret_cast<const uint4*>(w);
-      if (!g.z_tmem)
+      if (!z_tmem)
         *reinterpret_cast<uint4*>(smem + g.zg + off) = *reinterpret_cast<const uint4*>(z);
     }
   }
@@ -279,7 +281,7 @@ __global__ void __launch_bounds__((EW + 1) * 32, EW == 8 ? 2 : 1) res_kernel(con
     int kmax = min(8, g.H - k0);
     if (kmax > 0 && !SOMA_CHECK((size_t)(e * L.P + p0 + kmax) <= a.n_params, a.status)) kmax = 0;
     ProbeBits zb = {0u, 0u};
-    if (!g.z_tmem && kmax > 0 && do_z) zb = probe_bits(pk, p0, s.sparse);
+    if (!z_tmem && kmax > 0 && do_z) zb = probe_bits(pk, p0, s.sparse);
     __align__(16) __half w[8], z[8];
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
@@ -288,9 +290,9 @@ __global__ void __launch_bounds__((EW + 1) * 32, EW == 8 ? 2 : 1) res_kernel(con
       z[j] = ok ? z_half(zb, j) : __float2half_rn(0.f);
     }
     const uint32_t off = h * (128u * g.Hk * 2) + kmajor_offset(r, k0, g.Hk);
-    if (SOMA_CHECK(off + 16 <= 2u * 128u * g.Hk * 2 && (g.z_tmem || g.zo + off + 16 <= g.bytes), a.status)) {
+    if (SOMA_CHECK(off + 16 <= 2u * 128u * g.Hk * 2 && (z_tmem || g.zo + off + 16 <= g.bytes), a.status)) {
       *reinterpret_cast<uint4*>(smem + g.wo + off) = *reinterpret_cast<const uint4*>(w);
-      if (!g.z_tmem)
+      if (!z_tmem)
         *reinterpret_cast<uint4*>(smem + g.zo + off) = *reinterpret_cast<const uint4*>(z);
     }
   }
@@ -363,7 +365,7 @@ __global__ void __launch_bounds__((EW + 1) * 32, EW == 8 ? 2 : 1) res_kernel(con
   // probe tiles in tensor memory: thread = row (lane quarter w % 4), 8 columns
   // (16 k) per store; the warps of a quarter share the k steps.  Columns: the
   // gate tiles (K / 2 each), then the head halves (Hk / 2 each).
-  if (g.z_tmem && warp < EW) {
+  if (z_tmem && warp < EW) {
     const int r = 32 * q4 + lane;
     const uint32_t trow = tmem + ((uint32_t)(32 * q4) << 16) + g.zcol;
     const int gsteps = g.K / 16, hsteps = g.Hk / 16;
@@ -439,7 +441,7 @@ __global__ void __launch_bounds__((EW + 1) * 32, EW == 8 ? 2 : 1) res_kernel(con
     // columns; the descriptors stay in few instructions per MMA
     auto issue_tile = [&](uint32_t d, uint32_t wlo, uint32_t whi, uint32_t zlo, uint32_t zhi,
                           uint32_t zt, uint32_t ob, int steps) {
-      if (g.z_tmem) {
+      if (z_tmem) {
 #pragma unroll 4
         for (int k16 = 0; k16 < steps; ++k16) {
           const uint32_t ko = (uint32_t)k16 * 16, af = k16 > 0 ? 1u : 0u;
@@ -472,7 +474,7 @@ __global__ void __launch_bounds__((EW + 1) * 32, EW == 8 ? 2 : 1) res_kernel(con
       __syncwarp();
     };
     auto issue_head = [&](int t) {
-      const int buf = g.lag ? t & 1 : 0;
+      const int buf = kLag ? t & 1 : 0;
       const uint32_t hc = g.hcol + (uint32_t)buf * 4 * n2;
       if (!SOMA_CHECK(hc + 8u * g.Bp <= g.tmem_cols, a.status)) return;
       if (elect_one()) {
@@ -521,26 +523,26 @@ __global__ void __launch_bounds__((EW + 1) * 32, EW == 8 ? 2 : 1) res_kernel(con
       alive = res_wait(&ctl->op_ready, (uint32_t)t & 1u, abort, a.status);
       if (__any_sync(0xffffffffu, !alive)) break;
       tc_fence_after();
-      if (g.lag) {
+      if (kLag) {
         if (t + 1 < g.T) issue_gate(t + 1);
         issue_head(t);
       } else {
         issue_head(t);
-        if (!g.sep) {
+        if (!sep) {
           alive = res_wait(&ctl->acc_free, (uint32_t)t & 1u, abort, a.status);
           if (__any_sync(0xffffffffu, !alive)) break;
           tc_fence_after();
         }
         if (t + 1 < g.T) issue_gate(t + 1);
       }
-      if (t >= g.lag) {
-        const int tm = t - g.lag;
+      if (t >= kLag) {
+        const int tm = t - kLag;
         alive = res_wait(&ctl->red_full[tm & 1], (uint32_t)(tm >> 1) & 1u, abort, a.status);
         if (__any_sync(0xffffffffu, !alive)) break;
         merge(tm);
       }
     }
-    if (__all_sync(0xffffffffu, alive) && g.lag) {
+    if (__all_sync(0xffffffffu, alive) && kLag) {
       alive = res_wait(&ctl->red_full[(g.T - 1) & 1], (uint32_t)((g.T - 1) >> 1) & 1u, abort,
                        a.status);
       if (__all_sync(0xffffffffu, alive)) merge(g.T - 1);
@@ -601,7 +603,7 @@ __global__ void __launch_bounds__((EW + 1) * 32, EW == 8 ? 2 : 1) res_kernel(con
       }
       uint32_t wv[2][4], wd[2][4], zv[2][4], zd[2][4];
       load_groups(ng, tq, b0, wv, wd, zv, zd);
-      if (last && !g.sep) {  // the last read of the accumulator
+      if (last && !sep) {  // the last read of the accumulator
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(&ctl->acc_free);
@@ -662,8 +664,8 @@ __global__ void __launch_bounds__((EW + 1) * 32, EW == 8 ? 2 : 1) res_kernel(con
     // so after a wait that ran out the accumulators are read all the same (in
     // bounds, whatever they hold).
     auto head_epilogue = [&](int t) -> bool {
-      const uint32_t hb = g.lag ? (uint32_t)t & 1u : 0u;
-      const uint32_t par = g.lag ? (uint32_t)(t >> 1) & 1u : (uint32_t)t & 1u;
+      const uint32_t hb = kLag ? (uint32_t)t & 1u : 0u;
+      const uint32_t par = kLag ? (uint32_t)(t >> 1) & 1u : (uint32_t)t & 1u;
       const bool ok = res_wait(&ctl->head_bar[hb], par, abort, a.status);
       tc_fence_after();
       const uint32_t tq = tq0 + g.hcol + hb * 8u * g.Bp;
@@ -678,8 +680,6 @@ __global__ void __launch_bounds__((EW + 1) * 32, EW == 8 ? 2 : 1) res_kernel(con
         else
           head_groups(std::integral_constant<int, 1>(), t, c, tq, rd, yl, b0 + kStep >= g.Bp);
       }
-      // (a warp without a group)
-      if (!g.sep && 4 * sp >= g.Bp && lane == 0) mbar_arrive(&ctl->acc_free);
       __syncwarp();
       if (lane == 0) mbar_arrive(&ctl->red_full[t & 1]);
       return ok;
@@ -758,12 +758,12 @@ __global__ void __launch_bounds__((EW + 1) * 32, EW == 8 ? 2 : 1) res_kernel(con
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&ctl->op_ready);
-      if (t >= g.lag) {
-        alive = head_epilogue(t - g.lag);
+      if (t >= kLag) {
+        alive = head_epilogue(t - kLag);
         if (__any_sync(0xffffffffu, !alive)) break;
       }
     }
-    if (g.lag && __all_sync(0xffffffffu, alive)) head_epilogue(g.T - 1);
+    if (kLag && __all_sync(0xffffffffu, alive)) head_epilogue(g.T - 1);
   }
   tc_fence_before();
   __syncthreads();
