@@ -150,20 +150,14 @@ __device__ __forceinline__ int cst_lanes_of(const TcGeom& g) {
 
 // Shared-memory carve-up of one ring slot.
 struct StageLayout {
-  uint32_t a_off, b_off, b_src, b_bytes, bytes;
+  uint32_t a_off, b_off, bytes;
 };
 
 __host__ __device__ inline StageLayout stage_layout(const TcGeom& g) {
   StageLayout L;
   L.a_off = 0;
   L.b_off = kTileA;
-  // The window of the group tile that the perturbed copies and MMAs take, all of
-  // it, as run-time values: with them folded into the code the loader and the
-  // issuer come out slower (SOMA N=2 step 30.4 instead of 29.7 ms).  The
-  // unperturbed kernel does not use them (a group's own row blocks).
-  L.b_src = g.inf ? (uint32_t)(g.Bp / 8) * kSbo : 0u;
-  L.b_bytes = g.inf ? (uint32_t)(4 * g.Bp / 8) * kSbo : g.tileB;
-  L.bytes = (L.b_off + (g.inf ? g.tileB : L.b_bytes) + 1023u) & ~1023u;
+  L.bytes = (L.b_off + g.tileB + 1023u) & ~1023u;
   return L;
 }
 
@@ -1110,7 +1104,7 @@ tc_persistent_kernel(const TcArgs a) {
       const Phase ph = make_phase(a, t);
       // unperturbed: the row blocks the group has
       const uint32_t b_bytes =
-          INF ? (uint32_t)(inf_blocks(g, T.grp) * g.Bp / 8) * kSbo : SL.b_bytes;
+          INF ? (uint32_t)(inf_blocks(g, T.grp) * g.Bp / 8) * kSbo : g.tileB;
       // the operand rows other CTAs wrote (generic proxy) before the
       // fetcher's acquire are read here by bulk copies (async proxy)
       asm volatile("fence.proxy.async.global;" ::: "memory");
@@ -1130,7 +1124,7 @@ tc_persistent_kernel(const TcArgs a) {
             uint8_t* dst = lane == 0 ? slot + SL.a_off : slot + SL.b_off;
             const bool xs = !T.head && st < g.Sx;  // an embedding-part stage
             const uint8_t* src = lane == 0 ? T.a + (size_t)st * kTileA
-                                           : (xs ? T.bx : T.b) + (size_t)st * g.G * g.tileB + (INF ? 0u : SL.b_src);
+                                           : (xs ? T.bx : T.b) + (size_t)st * g.G * g.tileB;
             const uint32_t nb = lane == 0 ? kTileA : b_bytes;
             const uint8_t* gbase =
                 lane == 1 ? (xs ? a.xall : ph.op_in) : (T.head ? a.wo16 : a.w16);
@@ -1176,7 +1170,7 @@ tc_persistent_kernel(const TcArgs a) {
       const uint32_t a_lo0 = lo0 + (SL.a_off >> 4), b_lo0 = lo0 + (SL.b_off >> 4);
       const uint32_t grp_step = kSbo >> 4;                     // 8 operand rows
       // the W window starts at row Bp of the group tile (unperturbed: row 0)
-      const uint32_t w_row = INF ? 0u : (uint32_t)(g.Bp / 8) * grp_step - (SL.b_src >> 4);
+      const uint32_t w_row = INF ? 0u : (uint32_t)(g.Bp / 8) * grp_step;
       const uint32_t z1_row = (uint32_t)(4 * g.Bp / 8) * grp_step;
       const uint32_t dz1 = (uint32_t)(2 * g.Bp);
       RingPos<kStages> rp = {0u, 0u, 0u};
