@@ -409,6 +409,10 @@ int soma_body_adam_update(float* params, float* m, float* v, int n_experts, soma
                           int n_pert, int probe_kind, uint64_t seed, const uint64_t* steps,
                           int n_acc, const float* coef, soma_adam_config cfg, void* stream);
 
+/* soma_debug_body_streams: the streams (16-sequence chunks of a probe pair) that a
+ *   CTA of the body's forward runs, 1 or 2, for these sizes on a GPU of `sms` SMs;
+ *   0 if the sizes are invalid.  Host arithmetic only. */
+int soma_debug_body_streams(int n_experts, int n_pert, int batch, int sms);
 /* z_out device int8 [count]: body probe coordinates p0 .. p0 + count - 1
  * (p0 + count <= 2^30). */
 int soma_debug_body_probe(uint64_t seed, uint64_t step, int expert, int pert, soma_body_dims d,

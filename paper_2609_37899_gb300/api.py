@@ -147,6 +147,7 @@ def _open(path: str):
         _sig(L, "soma_body_adam_update", i32, [vp, vp, vp, i32, bd, i32, i32, u64,
                                                ctypes.POINTER(ctypes.c_uint64), i32, vp,
                                                soma_adam_config, vp])
+        _sig(L, "soma_debug_body_streams", i32, [i32, i32, i32, i32])
         _sig(L, "soma_debug_body_probe", i32, [u64, u64, i32, i32, bd, i32, i64, i64, vp, vp])
         _sig(L, "soma_checked_build", i32, [])
         _sig(L, "soma_debug_check_line", i32, [vp])

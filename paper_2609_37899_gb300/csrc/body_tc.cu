@@ -34,7 +34,7 @@
 // gates in tensor memory as A operands, Z of the MLP in shared memory),
 // operands and 160 accumulator columns, and meets the other stream nowhere.
 // Together they take 512 columns of tensor memory and 224 KB of shared memory.
-// With no more streams than SMs a CTA runs one.  After the barrier that
+// Where that saves no round of CTAs a CTA runs one (body_streams_per_cta).  After the barrier that
 // completes an operand, warp 0 of the stream issues the phase's MMAs; another
 // merges the decode's partials into the NLL while the next gates MMAs run.
 // Measured on GB300: the step of 256 bodies, 64 probes, 16 x 512 bytes, 570.7 ms
@@ -826,6 +826,20 @@ cudaError_t launch_streams(const BodyTcArgs& a, cudaStream_t stream) {
 
 }  // namespace
 
+// Two streams of one expert share a CTA where that takes fewer rounds of CTAs over
+// the SMs than one stream each.  An odd number of streams per expert leaves a CTA
+// half empty, and where that eats the rounds saved, one stream per CTA is the
+// shorter chain.  Measured (two streams -> one, T = 64): 100 experts x 3 probes of 16
+// sequences, 2 rounds either way, 1399 -> 1104 us; 200 x 1, 1192 -> 1096; 160 x 1 of
+// 48 sequences, 3 rounds against 4, 1969 -> 2142; 77 x 2, 1 against 2, 813 -> 1084;
+// 256 x 3, 4 against 6, 2788 -> 3236.
+int body_streams_per_cta(int n_experts, int n_pert, int B, int sms) {
+  const int64_t per_e = (int64_t)n_pert * ((B + kBp - 1) / kBp);
+  const int64_t one = (n_experts * per_e + sms - 1) / sms;
+  const int64_t two = (n_experts * ((per_e + 1) / 2) + sms - 1) / sms;
+  return two < one ? 2 : 1;
+}
+
 cudaError_t launch_body_tc(const float* params, const float* head, const uint8_t* bytes,
                            int n_experts, int blocks, int n_pert, int n_sign, int B, int T,
                            float eps, int sparse, uint64_t seed, uint64_t step, double* partial,
@@ -849,8 +863,8 @@ cudaError_t launch_body_tc(const float* params, const float* head, const uint8_t
   a.seed = seed;
   a.step = step;
   a.n_experts = n_experts;
-  // two streams per CTA once they do not all fit the SMs one by one
-  if ((int64_t)n_experts * n_pert * a.chunks > sm_count()) return launch_streams<2>(a, stream);
+  if (body_streams_per_cta(n_experts, n_pert, B, sm_count()) == 2)
+    return launch_streams<2>(a, stream);
   return launch_streams<1>(a, stream);
 }
 

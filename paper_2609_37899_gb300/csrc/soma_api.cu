@@ -826,6 +826,11 @@ int soma_body_adam_update(float* params, float* m, float* v, int n_experts, soma
                                       st, coef, h, (cudaStream_t)stream));
 }
 
+int soma_debug_body_streams(int n_experts, int n_pert, int batch, int sms) {
+  if (!body_sizes_ok(n_experts, n_pert, batch, 1) || sms < 1) return 0;
+  return body_streams_per_cta(n_experts, n_pert, batch, sms);
+}
+
 int soma_debug_body_probe(uint64_t seed, uint64_t step, int expert, int pert, soma_body_dims d,
                           int probe_kind, int64_t p0, int64_t count, int8_t* z_out,
                           void* stream) {

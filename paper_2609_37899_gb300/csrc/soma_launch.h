@@ -144,9 +144,10 @@ cudaError_t launch_probe_adam(float* params, float* m, float* v, int64_t P, int6
 // The paper's expert body (body.cu, body_tc.cu): width kBodyWidth, 1 <=
 // blocks <= kBodyMaxBlocks.  partial [N * n * n_sign][ceil(B / 16)] fp64 NLL sums.
 int body_rows_per_cta();
-// The antithetic forwards on the tensor cores (body_tc.cu): one CTA per
-// (expert, probe) pair and 16-sequence chunk, both signs in the
-// mean/difference form.
+// The antithetic forwards on the tensor cores (body_tc.cu): streams of one (expert,
+// probe) pair and 16-sequence chunk, both signs in the mean/difference form,
+// one or two of an expert per CTA.
+int body_streams_per_cta(int n_experts, int n_pert, int B, int sms);
 cudaError_t launch_body_tc(const float* params, const float* head, const uint8_t* bytes,
                            int n_experts, int blocks, int n_pert, int n_sign, int B, int T,
                            float eps, int sparse, uint64_t seed, uint64_t step, double* partial,
