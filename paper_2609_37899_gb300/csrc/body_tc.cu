@@ -129,6 +129,7 @@ static_assert(kTStream0 + kMaxStreams * kTStream <= kTmemCols, "tensor memory");
 
 struct BodyCtl {
   uint64_t mma_bar[kMaxStreams];   // the MMAs of a phase are done
+  uint64_t mma_done[kMaxStreams];  // all MMAs of the stream are
   uint32_t tmem_slot;
   volatile int abort;
 };
@@ -355,7 +356,10 @@ __global__ void __launch_bounds__(NS * kWarps * 32, 1) body_tc_kernel(const Body
   double* acc = reinterpret_cast<double*>(sm + S::acc);
 
   if (tid == 0) {
-    for (int k = 0; k < NS; ++k) mbar_init(&ctl->mma_bar[k], 1);
+    for (int k = 0; k < NS; ++k) {
+      mbar_init(&ctl->mma_bar[k], 1);
+      mbar_init(&ctl->mma_done[k], 1);
+    }
     ctl->abort = 0;
     mbar_fence_init();
   }
@@ -789,6 +793,13 @@ __global__ void __launch_bounds__(NS * kWarps * 32, 1) body_tc_kernel(const Body
           ylog[kBp + b] = k == 0 ? lm[0] : k == 1 ? lm[1] : k == 2 ? lm[2] : lm[3];
         }
       }
+    }
+    if (ew == kIssueWarp) {
+      // every MMA of the stream completes before its tensor memory is freed, also
+      // after a wait that ran out
+      if (elect_one()) mma_commit(&ctl->mma_done[st]);
+      __syncwarp();
+      mbar_wait(&ctl->mma_done[st], 0);
     }
     st_barrier();
     if (ew == kMergeWarp) {
