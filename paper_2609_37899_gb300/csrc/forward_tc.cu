@@ -1142,16 +1142,14 @@ tc_persistent_kernel(const TcArgs a) {
     }
     // The copies of the last stage of each slot land before the CTA exits
     // (earlier phases of a slot completed before its later copies were
-    // issued).  After an abort the copies issued so far are not tracked: the
-    // slot waits that failed above were bounded, and copies take
-    // microseconds against that bound.
-    if (done) {
+    // issued).  After an abort a slot's phase may lack the generators'
+    // arrivals and never complete: 4,096 polls, hundreds of microseconds, are
+    // then the time that the copies have to land.
 #pragma unroll
-      for (int q = 0; q < kStages; ++q) {
-        if ((int)gs <= q) continue;
-        const uint32_t last = gs - 1 - ((gs - 1 - (uint32_t)q) % kStages);  // last stage of slot q
-        mbar_wait(&ctl->full[q], (last / kStages) & 1u);
-      }
+    for (int q = 0; q < kStages; ++q) {
+      if ((int)gs <= q) continue;
+      const uint32_t last = gs - 1 - ((gs - 1 - (uint32_t)q) % kStages);  // last stage of slot q
+      mbar_wait(&ctl->full[q], (last / kStages) & 1u, done ? 1u << 22 : 1u << 12);
     }
   } else if (warp == kMmaWarp) {
     // ------------------------------------------------------------ MMA issuer
