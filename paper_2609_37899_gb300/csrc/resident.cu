@@ -33,10 +33,10 @@
 //    first, and the head epilogue of t - 1 runs under the gate MMAs of t + 1.
 // Measured on GB300 (a step, update included): 256 experts of E = 32, H = 48, 64
 // probes, 16 x 512 bytes: 161.9 ms with one CTA of 16 epilogue warps per SM and
-// a CTA barrier per timestep, 107.0 ms now (two per SM with a group of four
+// a CTA barrier per timestep, 105.9 ms now (two per SM with a group of four
 // sequences at a time 132 ms; groups in pairs 115; a commit per gate tile 110;
 // the MMA loops without a branch on the tile's place 107; the form's own parts
-// known at compile time, 15.8 -> 15.1 ms at T = 64).  One expert of E = 32,
+// known at compile time 105.9, at T = 64 15.8 -> 15.1).  One expert of E = 32,
 // H = 64, 8 probes, 4 x 64 bytes: 204 -> 159 us (the merge off the epilogue
 // warps, no barrier).  One MMA of this size occupies the tensor pipe about 46
 // cycles, so the 24 of a gate bound the latter's chain.
