@@ -129,7 +129,6 @@ static_assert(kTStream0 + kMaxStreams * kTStream <= kTmemCols, "tensor memory");
 
 struct BodyCtl {
   uint64_t mma_bar[kMaxStreams];   // the MMAs of a phase are done
-  uint64_t mma_done[kMaxStreams];  // all MMAs of the stream are
   uint32_t tmem_slot;
   volatile int abort;
 };
@@ -358,7 +357,6 @@ __global__ void __launch_bounds__(NS * kWarps * 32, 1) body_tc_kernel(const Body
   if (tid == 0) {
     for (int k = 0; k < NS; ++k) {
       mbar_init(&ctl->mma_bar[k], 1);
-      mbar_init(&ctl->mma_done[k], 1);
     }
     ctl->abort = 0;
     mbar_fence_init();
@@ -794,12 +792,13 @@ __global__ void __launch_bounds__(NS * kWarps * 32, 1) body_tc_kernel(const Body
         }
       }
     }
-    if (ew == kIssueWarp) {
-      // every MMA of the stream completes before its tensor memory is freed, also
-      // after a wait that ran out
-      if (elect_one()) mma_commit(&ctl->mma_done[st]);
-      __syncwarp();
-      mbar_wait(&ctl->mma_done[st], 0);
+    // The waits have completed every MMA, unless one ran out: then the batches still
+    // in flight complete before their tensor memory is freed.  Which phase the
+    // barrier is in is not known there, so waits on both parities take turns, 4,096
+    // polls (hundreds of microseconds) at most each.
+    if (ew == kIssueWarp && *abort) {
+#pragma unroll 1
+      for (uint32_t k = 0; k < 4; ++k) mbar_wait(mma_bar, (nph + k) & 1u, 1u << 12);
     }
     st_barrier();
     if (ew == kMergeWarp) {
