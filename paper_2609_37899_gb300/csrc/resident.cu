@@ -168,21 +168,6 @@ __device__ __forceinline__ __half z_half(const ProbeBits& b, int j) {
                              : __float2half_rn(0.f);
 }
 
-// A wait that times out records the status and sets the CTA's abort flag; one
-// that is still pending sees the flag within 64 polls and gives up too, so
-// every warp leaves its loop.
-__device__ __forceinline__ bool res_wait(uint64_t* bar, uint32_t parity, volatile int* abort,
-                                         int* status) {
-  if (mbar_try_wait(bar, parity)) return true;
-  for (uint32_t n = 1; n < (1u << 22); ++n) {
-    if ((n & 63u) == 0 && *abort) return false;
-    if (mbar_try_wait(bar, parity)) return true;
-  }
-  *abort = 1;
-  atomicCAS(status, 0, kStatusTimeout);
-  return false;
-}
-
 // fp16 pair word of z at offsets j, j + 1 of a run (natural bit order).
 __device__ __forceinline__ uint32_t z_pair_word(const ProbeBits& b, int j, int valid) {
   const __half lo = j < valid ? z_half(b, j) : __float2half_rn(0.f);
@@ -520,7 +505,7 @@ __global__ void __launch_bounds__((EW + 1) * 32, EW == 8 ? 2 : 1) res_kernel(con
     issue_gate(0);
     bool alive = true;
     for (int t = 0; t < g.T; ++t) {
-      alive = res_wait(&ctl->op_ready, (uint32_t)t & 1u, abort, a.status);
+      alive = lane_wait_inline(&ctl->op_ready, (uint32_t)t & 1u, abort, a.status);
       if (__any_sync(0xffffffffu, !alive)) break;
       tc_fence_after();
       if (kLag) {
@@ -529,7 +514,7 @@ __global__ void __launch_bounds__((EW + 1) * 32, EW == 8 ? 2 : 1) res_kernel(con
       } else {
         issue_head(t);
         if (!sep) {
-          alive = res_wait(&ctl->acc_free, (uint32_t)t & 1u, abort, a.status);
+          alive = lane_wait_inline(&ctl->acc_free, (uint32_t)t & 1u, abort, a.status);
           if (__any_sync(0xffffffffu, !alive)) break;
           tc_fence_after();
         }
@@ -537,14 +522,14 @@ __global__ void __launch_bounds__((EW + 1) * 32, EW == 8 ? 2 : 1) res_kernel(con
       }
       if (t >= kLag) {
         const int tm = t - kLag;
-        alive = res_wait(&ctl->red_full[tm & 1], (uint32_t)(tm >> 1) & 1u, abort, a.status);
+        alive = lane_wait_inline(&ctl->red_full[tm & 1], (uint32_t)(tm >> 1) & 1u, abort, a.status);
         if (__any_sync(0xffffffffu, !alive)) break;
         merge(tm);
       }
     }
     if (__all_sync(0xffffffffu, alive) && kLag) {
-      alive = res_wait(&ctl->red_full[(g.T - 1) & 1], (uint32_t)((g.T - 1) >> 1) & 1u, abort,
-                       a.status);
+      alive = lane_wait_inline(&ctl->red_full[(g.T - 1) & 1], (uint32_t)((g.T - 1) >> 1) & 1u,
+                               abort, a.status);
       if (__all_sync(0xffffffffu, alive)) merge(g.T - 1);
     }
 #pragma unroll
@@ -666,7 +651,7 @@ __global__ void __launch_bounds__((EW + 1) * 32, EW == 8 ? 2 : 1) res_kernel(con
     auto head_epilogue = [&](int t) -> bool {
       const uint32_t hb = kLag ? (uint32_t)t & 1u : 0u;
       const uint32_t par = kLag ? (uint32_t)(t >> 1) & 1u : (uint32_t)t & 1u;
-      const bool ok = res_wait(&ctl->head_bar[hb], par, abort, a.status);
+      const bool ok = lane_wait_inline(&ctl->head_bar[hb], par, abort, a.status);
       tc_fence_after();
       const uint32_t tq = tq0 + g.hcol + hb * 8u * g.Bp;
       float2* rd = red + (t & 1) * 16 * g.Bp;
@@ -727,7 +712,8 @@ __global__ void __launch_bounds__((EW + 1) * 32, EW == 8 ? 2 : 1) res_kernel(con
     for (int t = 0; t < g.T; ++t) {
       // the operand of t + 1: [x_{t+1} | h_t]
       uint8_t* opn = smem + g.op + (!(t & 1) ? g.opsz : 0u);
-      alive = res_wait(&ctl->gate_bar[EW == 8 && tile < g.MTg ? tile : 0], (uint32_t)t & 1u, abort, a.status);
+      alive = lane_wait_inline(&ctl->gate_bar[EW == 8 && tile < g.MTg ? tile : 0], (uint32_t)t & 1u,
+                               abort, a.status);
       if (__any_sync(0xffffffffu, !alive)) break;
       tc_fence_after();
       if (32 * tile + 8 * q4 < g.H) {  // the quarter holds units of the expert

@@ -98,8 +98,27 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity,
 // and sets the CTA's abort flag; one that is still pending sees the flag within
 // 64 polls and gives up too, so every warp leaves its loop.  A phase that is
 // already complete costs one poll and no read of the flag.
-// The polls after the first are a function of their own: in line they lengthen
-// the loops of every role (SOMA N=8 step at T = 128: 20.4 ms, 21.8 with them).
+//
+// The calling lane's answer.  After an abort the lanes of a warp may get
+// different ones: the caller votes before any lane leaves, for the others'
+// shuffles, votes and tensor-memory instructions would wait for it without a
+// bound.
+__device__ __forceinline__ bool lane_wait_inline(uint64_t* bar, uint32_t parity,
+                                                 volatile int* abort, int* status,
+                                                 uint32_t max_polls = 1u << 22) {
+  if (mbar_try_wait(bar, parity)) return true;
+  for (uint32_t n = 1; n < max_polls; ++n) {
+    if ((n & 63u) == 0 && *abort) return false;
+    if (mbar_try_wait(bar, parity)) return true;
+  }
+  *abort = 1;
+  atomicCAS(status, 0, kStatusTimeout);
+  return false;
+}
+
+// The same with the polls after the first in a function of their own: in line
+// they lengthen the loops of every role (SOMA N=8 step at T = 128: 20.4 ms, 21.8
+// with them).
 __device__ __noinline__ inline bool lane_wait_more(uint64_t* bar, uint32_t parity,
                                                    volatile int* abort, int* status,
                                                    uint32_t max_polls) {
@@ -114,11 +133,6 @@ __device__ __noinline__ inline bool lane_wait_more(uint64_t* bar, uint32_t parit
   }
   return done;
 }
-
-// The calling lane's answer.  After an abort the lanes of a warp may get
-// different ones: the caller votes before any lane leaves, for the others'
-// shuffles, votes and tensor-memory instructions would wait for it without a
-// bound.
 __device__ __forceinline__ bool lane_wait(uint64_t* bar, uint32_t parity, volatile int* abort,
                                           int* status, uint32_t max_polls = 1u << 22) {
   return mbar_try_wait(bar, parity) || lane_wait_more(bar, parity, abort, status, max_polls);
