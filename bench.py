@@ -47,9 +47,19 @@ TRAFFIC = {
     # profiles/tc_persistent_kernel_soma_n2.md: one persistent launch of the
     # SOMA N=2 shapes at T=16 (17 phases) captured; per phase, scaled by the
     # T + 1 phases of a launch
-    "soma_n2": {"bytes_per_phase": (2200.845824e6 + 870.040064e6) / 17,
+    "soma_n2": {"bytes_per_phase": (2201.425408e6 + 870.437888e6) / 17,
                 "files": ["forward_tc.cu", "tc_primitives.cuh", "soma_device.cuh"],
-                "source_hash": "ee8ef0435f95da87"},
+                "source_hash": "5f9762c0964999a7"},
+    # profiles/res_kernel_soma_n256.md: one launch at T=128; a launch reads the
+    # parameters once and N B (T + 1) bytes of sequences
+    "soma_n256": {"bytes_per_launch": 37.815808e6 + 51712, "seq_len": 128, "batch": 256 * 16,
+                  "files": ["resident.cu", "tc_primitives.cuh", "soma_device.cuh"],
+                  "source_hash": "3ff3c380f4725d2d"},
+    # profiles/body_tc_kernel_body_n256.md: one launch at T=96, likewise
+    "body_n256": {"bytes_per_launch": 34.250240e6, "seq_len": 96, "batch": 256 * 16,
+                  "files": ["body_tc.cu", "body_device.cuh", "tc_primitives.cuh",
+                            "soma_device.cuh"],
+                  "source_hash": "612f7513ee96c416"},
 }
 
 
@@ -311,13 +321,14 @@ def source_hash(files):
 def launch_traffic(config, T):
     """DRAM bytes of one launch of the dominant kernel at sequence length T,
     or None when the sources changed since the capture.  A per-phase figure
-    scales to the T + 1 phases of one persistent launch."""
+    scales to the T + 1 phases of one persistent launch; a resident launch
+    reads one byte more per sequence and timestep than the captured one."""
     tr = TRAFFIC.get(config)
     if not tr or tr["source_hash"] != source_hash(tr["files"]):
         return None
     if "bytes_per_phase" in tr:
         return tr["bytes_per_phase"] * (T + 1)
-    return tr["bytes_per_launch"]
+    return tr["bytes_per_launch"] + tr.get("batch", 0) * (T - tr.get("seq_len", T))
 
 
 def our_arm(args):

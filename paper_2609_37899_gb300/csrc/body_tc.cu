@@ -34,17 +34,18 @@
 // gates in tensor memory as A operands, Z of the MLP in shared memory),
 // operands and 160 accumulator columns, and meets the other stream nowhere.
 // Together they take 512 columns of tensor memory and 224 KB of shared memory.
-// Where that saves no round of CTAs a CTA runs one (body_streams_per_cta).  After the barrier that
-// completes an operand, warp 0 of the stream issues the phase's MMAs; another
-// merges the decode's partials into the NLL while the next gates MMAs run.
+// Where that saves no round of CTAs a CTA runs one (body_streams_per_cta).
+// After the barrier that completes an operand, warp 0 of the stream issues the
+// phase's MMAs; another merges the decode's partials into the NLL while the next
+// gates MMAs run.
 // Measured on GB300: the step of 256 bodies, 64 probes, 16 x 512 bytes, 570.7 ms
 // with one stream per SM (16 epilogue warps, a CTA barrier per phase), 476 with
 // two of 8 epilogue warps and an MMA warp each, 357 with two of 16 warps that
-// issue their own MMAs, 333 ms now (offsets and pairs precomputed, LN on half
+// issue their own MMAs, 331 ms now (offsets and pairs precomputed, LN on half
 // of the warps).  Alone on its SM a stream takes about 15,000 cycles per
 // timestep: MMA batches 5,000, GELU 2,300 (its erff), LN 2,500, cells and decode
 // 2,600 and the rest barriers and tensor-memory reads; two together 24,000,
-// 67 % of the issue slots busy.
+// 64 % of the issue slots busy.
 //
 // Precision.  With plain fp16 operands the losses were off by up to ~2e-4
 // nats/byte and the coefficients by ~1-2% on small batches: the rounding of

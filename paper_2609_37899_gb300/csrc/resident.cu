@@ -37,7 +37,7 @@
 // sequences at a time 132 ms; groups in pairs 115; a commit per gate tile 110;
 // the MMA loops without a branch on the tile's place 107; the form's own parts
 // known at compile time 105.9, at T = 64 15.8 -> 15.1).  One expert of E = 32,
-// H = 64, 8 probes, 4 x 64 bytes: 204 -> 159 us (the merge off the epilogue
+// H = 64, 8 probes, 4 x 64 bytes: 207 -> 156 us (the merge off the epilogue
 // warps, no barrier).  One MMA of this size occupies the tensor pipe about 46
 // cycles, so the 24 of a gate bound the latter's chain.
 // The shape limits are checked by res_supported(); other experts use the
